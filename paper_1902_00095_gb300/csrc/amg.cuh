@@ -232,6 +232,13 @@ void chebyshev_apply(const Level& v, const TV* val, const TV* dinv, int degree, 
 DevCSR csr_product(const DevCSR& A, const DevCSR& B, Pool& pool, Pool& scratch,
                    cudaStream_t s);
 void csr_product_numeric(const DevCSR& A, const DevCSR& B, const DevCSR& C, cudaStream_t s);
+// Truncated (pmax >= 1 weights per row) classical or extended+i interpolation
+// P of level operator A (amg_interp.cu); P's arrays from `pool`. Returns false
+// when a row is past its capacities (nothing usable written).
+bool truncated_interpolation(const DevCSR& A, bool extended, int sms, const int* dpos,
+                             const unsigned char* strong, const signed char* state,
+                             const int* cidx, int nc, int pmax, Pool& pool, Pool& scratch,
+                             DevCSR& P, cudaStream_t s);
 void csr_transpose_positions(const DevCSR& A, int* tpos, int* err, cudaStream_t s);
 
 }  // namespace tp

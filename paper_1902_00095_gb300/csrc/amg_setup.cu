@@ -7,7 +7,7 @@
 // split is PMIS with seeded tie-breaks and the interpolation is classical or
 // its distance-two extended+i form; all structure-deciding arithmetic uses
 // __dmul_rn / __dadd_rn / __ddiv_rn in a fixed ascending-column order.
-#include "amg.cuh"
+#include "amg_dev.cuh"
 #include <chrono>
 #include <cmath>
 #include <algorithm>
@@ -15,8 +15,6 @@
 namespace tp {
 
 namespace {
-
-constexpr signed char kC = 1, kF = -1, kU = 0;
 
 int setup_sms();
 long long resident_threads();
@@ -297,30 +295,6 @@ __global__ void k_classical_count(int n, const int* __restrict__ rp, const int* 
   for (int e = rp[i]; e < rp[i + 1]; ++e)
     if (strong[e] && state[col[e]] == kC) ++c;
   cnt[i] = c;
-}
-
-// sign class of a_kk for opposite(): 0 when a_kk is zero or NaN (never
-// opposite), 1 positive, 2 negative (one byte per entry in shared memory
-// instead of the value)
-__device__ __forceinline__ unsigned char sign_class(double d) {
-  const unsigned long long ud = (unsigned long long)__double_as_longlong(d);
-  const unsigned long long md = ud & 0x7fffffffffffffffull;
-  if (md == 0 || md > 0x7ff0000000000000ull) return 0;
-  return (unsigned char)(1 + (ud >> 63));
-}
-
-// opposite(a, d) with d given by its sign class
-__device__ __forceinline__ bool opposite_class(double a, unsigned char dc) {
-  const unsigned long long ua = (unsigned long long)__double_as_longlong(a);
-  const unsigned long long ma = ua & 0x7fffffffffffffffull;
-  return dc != 0 && ma != 0 && ma <= 0x7ff0000000000000ull &&
-         (unsigned)(ua >> 63) != (unsigned)(dc - 1);
-}
-
-// an FP64 value is non-zero (either sign, or NaN), tested on its bits: FP64
-// compares would take the FP64 pipe
-__device__ __forceinline__ bool nonzero_bits(double v) {
-  return ((unsigned long long)__double_as_longlong(v) << 1) != 0;
 }
 
 // rows longer than kClsShort are filled by a warp (k_classical_fill_warp)
@@ -2240,13 +2214,23 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
       cur.cf = nullptr;  // this level becomes the coarsest
       break;
     }
-    // interpolation
+    // interpolation: in one pass when it is truncated, else (and for levels
+    // with a row past that pass's capacities) sets, weights and truncation
+    // by kernels of their own
     DevCSR P;
-    P.n = n;
-    P.m = nc;
-    P.rowptr = pool.alloc<int>(n + 1);
-    int* cnt = scratch.alloc<int>(n + 1);
-    if (opts.interp == 0) {
+    const bool one_pass =
+        opts.pmax > 0 && truncated_interpolation(A, opts.interp != 0, setup_sms(), cur.dpos,
+                                                 cur.strong, cur.cf, cidx, nc, opts.pmax, pool,
+                                                 scratch, P, s);
+    int* cnt = nullptr;
+    if (!one_pass) {
+      P.n = n;
+      P.m = nc;
+      P.rowptr = pool.alloc<int>(n + 1);
+      cnt = scratch.alloc<int>(n + 1);
+    }
+    if (one_pass) {
+    } else if (opts.interp == 0) {
       k_classical_count<<<grid_for(n), kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.cf,
                                                        cnt);
       TP_LAUNCH_CHECK();
@@ -2294,7 +2278,7 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
           P.col, P.val);
       TP_LAUNCH_CHECK();
     }
-    if (opts.pmax > 0) {
+    if (!one_pass && opts.pmax > 0) {
       DevCSR T;
       T.n = n;
       T.m = nc;

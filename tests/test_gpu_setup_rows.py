@@ -1,0 +1,72 @@
+"""AMG setup kernels at the edges of their row classes: every level's operator,
+C/F split and interpolation bit for bit against the oracle, on matrices whose
+rows reach past each class's capacities (row length, strong neighbours, set
+size, products), and with and without truncation."""
+import numpy as np
+import pytest
+
+from oracle import amg as oamg
+
+pytestmark = pytest.mark.gpu
+
+thermo = pytest.importorskip("paper_1902_00095_gb300.thermo")
+
+
+def graph_matrix(n, degree, seed, hubs=0, positive=0.0):
+    """Diagonally dominant matrix on a random symmetric graph of mean degree
+    `degree`, non-symmetric values, a share `positive` of them positive;
+    `hubs` rows connected to every other row."""
+    rng = np.random.default_rng(seed)
+    m = n * degree // 2
+    i, j = rng.integers(0, n, m), rng.integers(0, n, m)
+    near = rng.random(m) < 0.7  # most edges short, so that sets overlap
+    j = np.where(near, (i + rng.integers(1, 2 + 2 * degree, m)) % n, j)
+    pairs = {(min(a, b), max(a, b)) for a, b in zip(i, j) if a != b}
+    for h in range(hubs):
+        pairs |= {(min(h, b), max(h, b)) for b in range(n) if b != h}
+    pairs = np.array(sorted(pairs))
+    rows = np.concatenate([pairs[:, 0], pairs[:, 1], np.arange(n)])
+    cols = np.concatenate([pairs[:, 1], pairs[:, 0], np.arange(n)])
+    vals = -10.0 ** rng.uniform(-2.0, 0.0, rows.size)
+    vals[rng.random(rows.size) < positive] *= -0.1
+    order = np.lexsort((cols, rows))
+    rows, cols, vals = rows[order], cols[order].astype(np.int32), vals[order]
+    rowptr = np.zeros(n + 1, np.int64)
+    rowptr[1:] = np.cumsum(np.bincount(rows, minlength=n))
+    off = np.where(rows != cols, np.abs(vals), 0.0)
+    diag = rows == cols
+    vals[diag] = 1.02 * np.add.reduceat(off, rowptr[:-1]) + 1e-3
+    return rowptr, cols, vals
+
+
+def compare(A, interp, pmax, levels):
+    g = thermo.AMG(*A, interp=interp, pmax=pmax, max_levels=levels, coarse_size=20, seed=3)
+    h = oamg.setup(A, seed=3, coarse_size=20, max_levels=levels, pmax=pmax,
+                   interp="ext+i" if interp else "classical")
+    n, nnz = g.info()
+    assert list(n) == [lev["n"] for lev in h["levels"]]
+    for l, lev in enumerate(h["levels"]):
+        e = g.export_level(l)
+        for a, b in zip(e["A"], lev["A"]):
+            assert np.array_equal(a, b), l
+        if "P" in lev:
+            assert np.array_equal(e["cf"], lev["cf"]), l
+            for a, b in zip(e["P"], lev["P"]):
+                assert np.array_equal(a, b), l
+    g.close()
+
+
+# degree 6: rows of the 8-lane class and a few past it; 40: the 16-lane class;
+# 110 and 220: past its row length, neighbours and lists; 30 with hub rows of
+# 1500 entries: past the one-pass kernels' last capacities
+@pytest.mark.parametrize("n,degree,hubs", [(900, 6, 0), (25, 6, 0), (700, 40, 0), (900, 110, 0),
+                                           (1000, 220, 0), (1500, 30, 2)])
+@pytest.mark.parametrize("interp", [0, 1])
+def test_interpolation_and_galerkin_rows_are_bit_exact(n, degree, hubs, interp):
+    compare(graph_matrix(n, degree, seed=n + degree, hubs=hubs, positive=0.1), interp, 4, 3)
+
+
+@pytest.mark.parametrize("pmax", [1, 3, 16, 0])
+@pytest.mark.parametrize("interp", [0, 1])
+def test_interpolation_widths_are_bit_exact(pmax, interp):
+    compare(graph_matrix(600, 14, seed=pmax, positive=0.2), interp, pmax, 2)
