@@ -231,7 +231,8 @@ void chebyshev_apply(const Level& v, const TV* val, const TV* dinv, int degree, 
 // `pool`), and the numeric-only recomputation of C's values on its pattern.
 DevCSR csr_product(const DevCSR& A, const DevCSR& B, Pool& pool, Pool& scratch,
                    cudaStream_t s);
-void csr_product_numeric(const DevCSR& A, const DevCSR& B, const DevCSR& C, cudaStream_t s);
+void csr_product_numeric(const DevCSR& A, const DevCSR& B, const DevCSR& C, Pool& scratch,
+                         cudaStream_t s);
 // Truncated (pmax >= 1 weights per row) classical or extended+i interpolation
 // P of level operator A (amg_interp.cu); P's arrays from `pool`. Returns false
 // when a row is past its capacities (nothing usable written).

@@ -33,4 +33,15 @@ __device__ __forceinline__ bool nonzero_bits(double v) {
   return ((unsigned long long)__double_as_longlong(v) << 1) != 0;
 }
 
+// index of key in a[lo, hi) (ascending), or -1
+__device__ __forceinline__ int find_in(const int* __restrict__ a, int lo, int hi, int key) {
+  int h = hi;
+  while (lo < hi) {
+    int mid = (lo + hi) >> 1;
+    if (a[mid] < key) lo = mid + 1;
+    else hi = mid;
+  }
+  return (lo < h && a[lo] == key) ? lo : -1;
+}
+
 }  // namespace tp

@@ -19,17 +19,6 @@ namespace {
 int setup_sms();
 long long resident_threads();
 
-// index of key in a[lo, hi) (ascending), or -1
-__device__ __forceinline__ int find_in(const int* __restrict__ a, int lo, int hi, int key) {
-  int h = hi;
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (a[mid] < key) lo = mid + 1;
-    else hi = mid;
-  }
-  return (lo < h && a[lo] == key) ? lo : -1;
-}
-
 // (d > 0 && a < 0) || (d < 0 && a > 0), decided on the bit patterns: both
 // non-zero, neither NaN, signs differ. Integer operations instead of FP64
 // comparisons, which on this part share the FP64 pipe (2 per clock per SM)
@@ -936,618 +925,6 @@ __global__ void k_rank_rows_warp(int n, const int* __restrict__ rp, const int* _
   }
 }
 
-// ------------------------------------------------------------- SpGEMM C = A B
-// Upper bound (product count) of every row of C = A B; rows too long for
-// the thread-per-row kernel are listed for the warp kernel (kSpShort < ub <
-// kSpCap) or the block kernel (ub >= kSpCap), so those visit only their rows.
-// The list order is not deterministic; each row's result is.
-__global__ void k_spgemm_ub(int n, const int* __restrict__ Arp, const int* __restrict__ Acol,
-                            const int* __restrict__ Brp, int* __restrict__ ub,
-                            int* __restrict__ wlist, int* __restrict__ blist,
-                            int* __restrict__ counts);
-
-// Row i of C: products a_ik * b_kj in ascending k (row i of A) then ascending
-// j (row k of B); each column's sum starts at 0.0 and adds them in that
-// order. Columns kept sorted by insertion. This thread-per-row form takes
-// the rows with at most kSpShort products and more than kSpMerge entries of
-// A (k_spgemm_rows_merge the rows with fewer, k_spgemm_rows_warp the rows
-// with more products).
-constexpr int kSpShort = 96;
-constexpr int kSpMerge = 8;  // rows of A with at most this many entries: k-way merge
-
-// The rows of k_spgemm_rows whose row of A has at most kSpMerge entries (a
-// 7-point operator times P): a merge of the (sorted) rows of B of the row's
-// entries, heads in registers. Each column comes out once, in order, its
-// products added in ascending entry order from 0.0 (the canonical order),
-// with no sorted-list insertion in memory. A kernel of its own: its
-// registers would cost the insertion form occupancy.
-__global__ void k_spgemm_rows_merge(int n, const int* __restrict__ Arp,
-                                    const int* __restrict__ Acol, const double* __restrict__ Aval,
-                                    const int* __restrict__ Brp, const int* __restrict__ Bcol,
-                                    const double* __restrict__ Bval, const int* __restrict__ off,
-                                    const int* __restrict__ ub, int* __restrict__ ccol,
-                                    double* __restrict__ cval, int* __restrict__ cnt) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || ub[i] > kSpShort) return;
-  const int a0 = Arp[i], na = Arp[i + 1] - a0;
-  if (na > kSpMerge) return;
-  int* cc = ccol + off[i];
-  double* cv = cval + off[i];
-  // a merge of the (sorted) rows of B of the row's entries, heads in
-  // registers: each column comes out once, in order, its products added
-  // in ascending entry order from 0.0 (the canonical order), with no
-  // sorted-list insertion in memory (rows of a 7-point operator times P)
-  int f[kSpMerge], fe[kSpMerge], hc[kSpMerge];
-  double av[kSpMerge];
-#pragma unroll
-  for (int k = 0; k < kSpMerge; ++k) {
-    f[k] = fe[k] = 0;
-    hc[k] = 0x7fffffff;
-    av[k] = 0.0;
-    if (k < na) {
-      const int kk = Acol[a0 + k];
-      av[k] = Aval[a0 + k];
-      f[k] = Brp[kk];
-      fe[k] = Brp[kk + 1];
-      if (f[k] < fe[k]) hc[k] = Bcol[f[k]];
-    }
-  }
-  int u = 0;
-  while (true) {
-    int m = 0x7fffffff;
-#pragma unroll
-    for (int k = 0; k < kSpMerge; ++k) m = min(m, hc[k]);
-    if (m == 0x7fffffff) break;
-    double sum = 0.0;
-#pragma unroll
-    for (int k = 0; k < kSpMerge; ++k)
-      if (hc[k] == m) {
-        sum = __dadd_rn(sum, __dmul_rn(av[k], Bval[f[k]]));
-        ++f[k];
-        hc[k] = f[k] < fe[k] ? Bcol[f[k]] : 0x7fffffff;
-      }
-    cc[u] = m;
-    cv[u] = sum;
-    ++u;
-  }
-  cnt[i] = u;
-}
-
-__global__ void k_spgemm_rows(int n, const int* __restrict__ Arp, const int* __restrict__ Acol,
-                              const double* __restrict__ Aval, const int* __restrict__ Brp,
-                              const int* __restrict__ Bcol, const double* __restrict__ Bval,
-                              const int* __restrict__ off, const int* __restrict__ ub,
-                              int* __restrict__ ccol, double* __restrict__ cval,
-                              int* __restrict__ cnt) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || ub[i] > kSpShort) return;
-  int* cc = ccol + off[i];
-  double* cv = cval + off[i];
-  if (Arp[i + 1] - Arp[i] <= kSpMerge) return;  // k_spgemm_rows_merge
-  int u = 0;
-  for (int e = Arp[i]; e < Arp[i + 1]; ++e) {
-    const int k = Acol[e];
-    const double a = Aval[e];
-    for (int f = Brp[k]; f < Brp[k + 1]; ++f) {
-      const int j = Bcol[f];
-      const double prod = __dmul_rn(a, Bval[f]);
-      int lo = 0, hi = u;
-      while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (cc[mid] < j) lo = mid + 1;
-        else hi = mid;
-      }
-      if (lo < u && cc[lo] == j) {
-        cv[lo] = __dadd_rn(cv[lo], prod);
-      } else {
-        for (int q = u; q > lo; --q) {
-          cc[q] = cc[q - 1];
-          cv[q] = cv[q - 1];
-        }
-        cc[lo] = j;
-        cv[lo] = __dadd_rn(0.0, prod);
-        ++u;
-      }
-    }
-  }
-  cnt[i] = u;
-}
-
-// Products whose result has few columns (m <= kDenseCap: the Galerkin
-// products of coarse levels): one warp per row accumulates into a dense
-// shared-memory row. The entries of row i of A are visited in order and the
-// lanes split row k of B (whose columns are distinct), so every column's sum
-// still starts at 0.0 and adds its products in ascending k: the canonical
-// order. Touched columns are flagged and compacted in column order.
-constexpr int kDenseCap = 2048;
-constexpr int kDenseWarps = 4;
-constexpr size_t kDenseSmem = (size_t)kDenseWarps * kDenseCap * (sizeof(double) + 1);
-
-__global__ void __launch_bounds__(32 * kDenseWarps) k_spgemm_dense(
-    int n, int m, const int* __restrict__ Arp, const int* __restrict__ Acol,
-    const double* __restrict__ Aval, const int* __restrict__ Brp, const int* __restrict__ Bcol,
-    const double* __restrict__ Bval, const int* __restrict__ off, int* __restrict__ ccol,
-    double* __restrict__ cval, int* __restrict__ cnt) {
-  extern __shared__ double s_dense[];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned below = (1u << lane) - 1u;
-  double* acc = s_dense + (size_t)w * m;
-  unsigned char* flg = reinterpret_cast<unsigned char*>(s_dense + (size_t)kDenseWarps * m) +
-                       (size_t)w * m;
-  for (int i = blockIdx.x * kDenseWarps + w; i < n; i += gridDim.x * kDenseWarps) {
-    for (int j = lane; j < m; j += 32) {
-      acc[j] = 0.0;
-      flg[j] = 0;
-    }
-    __syncwarp();
-    for (int e = Arp[i]; e < Arp[i + 1]; ++e) {
-      const int k = Acol[e];
-      const double a = Aval[e];
-      for (int f = Brp[k] + lane; f < Brp[k + 1]; f += 32) {
-        const int j = Bcol[f];
-        acc[j] = __dadd_rn(acc[j], __dmul_rn(a, Bval[f]));
-        flg[j] = 1;
-      }
-      __syncwarp();
-    }
-    int* cc = ccol + off[i];
-    double* cv = cval + off[i];
-    int base = 0;
-    for (int j0 = 0; j0 < m; j0 += 32) {
-      const int j = j0 + lane;
-      const bool has = j < m && flg[j];
-      const unsigned hm = __ballot_sync(0xffffffffu, has);
-      if (has) {
-        cc[base + __popc(hm & below)] = j;
-        cv[base + __popc(hm & below)] = acc[j];
-      }
-      base += __popc(hm);
-    }
-    if (lane == 0) cnt[i] = base;
-    __syncwarp();
-  }
-}
-
-// Warp-per-row variant of k_spgemm_rows with the same summation order. The
-// warp walks row i of A in ascending k; for each k its lanes take distinct
-// entries of row k of B (whose columns are distinct), so no two lanes update
-// the same column at once, and a __syncwarp between k's keeps every
-// column's additions in ascending k, each sum starting at 0.0: the canonical
-// order. Columns find their accumulator through an open-addressing hash
-// table in shared memory (linear probing, at least twice as many slots as
-// products, so an empty slot always exists); the distinct columns are then
-// sorted by a warp bitonic sort of (column << 32 | slot) keys and written
-// in ascending order. Each batch of 32 entries of row i of A (column k,
-// value, row k's extent in B) is loaded by the warp at once, so a step over
-// k waits for one round trip (row k of B), not three. Rows with fewer than
-// kSpMid products use tables of kSpMid slots (four warps per block), rows
-// up to kSpCap tables of kSpCap slots (two warps); longer rows go to the
-// block kernel.
-constexpr int kSpMid = 512;
-constexpr int kSpCap = 1024;
-
-__global__ void k_spgemm_ub(int n, const int* __restrict__ Arp, const int* __restrict__ Acol,
-                            const int* __restrict__ Brp, int* __restrict__ ub,
-                            int* __restrict__ wlist, int* __restrict__ blist,
-                            int* __restrict__ counts) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int u = 0;
-  for (int e = Arp[i]; e < Arp[i + 1]; ++e) {
-    int k = Acol[e];
-    u += Brp[k + 1] - Brp[k];
-  }
-  ub[i] = u;
-  if (u >= kSpCap) blist[atomicAdd(&counts[1], 1)] = i;
-  else if (u >= kSpMid) wlist[n - 1 - atomicAdd(&counts[2], 1)] = i;
-  else if (u > kSpShort) wlist[atomicAdd(&counts[0], 1)] = i;
-}
-
-__device__ void spgemm_row_serial(int i, const int* __restrict__ Arp, const int* __restrict__ Acol,
-                                  const double* __restrict__ Aval, const int* __restrict__ Brp,
-                                  const int* __restrict__ Bcol, const double* __restrict__ Bval,
-                                  int* __restrict__ cc, double* __restrict__ cv, int* __restrict__ cnt) {
-  int u = 0;
-  for (int e = Arp[i]; e < Arp[i + 1]; ++e) {
-    const int k = Acol[e];
-    const double a = Aval[e];
-    for (int f = Brp[k]; f < Brp[k + 1]; ++f) {
-      const int j = Bcol[f];
-      const double prod = __dmul_rn(a, Bval[f]);
-      int lo = 0, hi = u;
-      while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (cc[mid] < j) lo = mid + 1;
-        else hi = mid;
-      }
-      if (lo < u && cc[lo] == j) {
-        cv[lo] = __dadd_rn(cv[lo], prod);
-      } else {
-        for (int q = u; q > lo; --q) {
-          cc[q] = cc[q - 1];
-          cv[q] = cv[q - 1];
-        }
-        cc[lo] = j;
-        cv[lo] = __dadd_rn(0.0, prod);
-        ++u;
-      }
-    }
-  }
-  cnt[i] = u;
-}
-
-// one warp: row i of C = A B through a shared-memory hash table of
-// 2^k >= 2 ex slots (hkey/hval, at most `tcap`), then the distinct columns
-// sorted in skey (capacity tcap)
-__device__ void spgemm_row_hash(int i, int ex, int lane, int tcap, const int* __restrict__ Arp,
-                                const int* __restrict__ Acol, const double* __restrict__ Aval,
-                                const int* __restrict__ Brp, const int* __restrict__ Bcol,
-                                const double* __restrict__ Bval, int* hkey, double* hval,
-                                unsigned long long* skey, int* __restrict__ cc,
-                                double* __restrict__ cv, int* __restrict__ cnt) {
-  int bits = 5;
-  while ((1 << bits) < 2 * ex && (1 << bits) < tcap) ++bits;
-  const int cap = 1 << bits;
-  const unsigned below = (1u << lane) - 1u;
-  for (int q = lane; q < cap; q += 32) hkey[q] = -1;
-  __syncwarp();
-  // 1. accumulate in canonical order: every column's sum starts at 0.0 and
-  // takes its products in ascending e. Rows of fewer than kSpMid products
-  // whose rows of B are short (fewer than 16 products per entry of A on
-  // average, as in A P; measured faster there, slower on the rows of
-  // kSpMid-kSpCap products of R (A P)) take the
-  // next 32 products of the row in sequence order per step (entry e of row i
-  // of A, then the row of B): lanes claim their column's slot, and lanes of
-  // one step that share a column (at most one product per entry e, so lane
-  // order is entry order) are added by the lowest of them in lane order onto
-  // the sum of the earlier steps. Other rows take one entry of A per step,
-  // its row of B split over the lanes (distinct columns).
-  for (int q = lane; q < cap; q += 32) hval[q] = 0.0;
-  __syncwarp();
-  double* sprod = reinterpret_cast<double*>(skey);  // 32 staged products
-  const int a0 = Arp[i], a1 = Arp[i + 1];
-  if (tcap <= kSpMid && ex < 16 * (a1 - a0)) {
-    for (int e0 = a0; e0 < a1; e0 += 32) {
-      const int e = e0 + lane;
-      double a = 0.0;
-      int fb = 0, len = 0;
-      if (e < a1) {
-        const int k = Acol[e];
-        a = Aval[e];
-        fb = Brp[k];
-        len = Brp[k + 1] - fb;
-      }
-      int incl = len;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const int excl = incl - len;
-      const int total = __shfl_sync(0xffffffffu, incl, 31);
-      for (int p0 = 0; p0 < total; p0 += 32) {
-        const int p = p0 + lane;
-        // the entry holding position p: the last lane with excl <= p
-        int lo = 0;
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1) {
-          const int cand = lo + step;
-          if (__shfl_sync(0xffffffffu, excl, cand) <= p) lo = cand;
-        }
-        const int se = __shfl_sync(0xffffffffu, excl, lo);
-        const int sf = __shfl_sync(0xffffffffu, fb, lo);
-        const double sa = __shfl_sync(0xffffffffu, a, lo);
-        int slot = -1 - lane;  // distinct for lanes without a product
-        double prod = 0.0;
-        if (p < total) {
-          const int f = sf + (p - se);
-          const int j = Bcol[f];
-          prod = __dmul_rn(sa, Bval[f]);
-          unsigned h = ((unsigned)j * 0x9E3779B1u) >> (32 - bits);
-          for (int probe = 0; probe < cap; ++probe) {
-            const int prev = atomicCAS(&hkey[h], -1, j);
-            if (prev == -1 || prev == j) {
-              slot = (int)h;
-              break;
-            }
-            h = (h + 1) & (unsigned)(cap - 1);
-          }
-        }
-        sprod[lane] = prod;
-        const unsigned grp = __match_any_sync(0xffffffffu, slot);
-        __syncwarp();
-        if (slot >= 0 && (grp & below) == 0) {
-          double v = hval[slot];
-          for (unsigned g = grp; g; g &= g - 1u) v = __dadd_rn(v, sprod[__ffs(g) - 1]);
-          hval[slot] = v;
-        }
-        __syncwarp();
-      }
-    }
-  } else {
-    for (int e0 = a0; e0 < a1; e0 += 32) {
-      const int e = e0 + lane;
-      double a = 0.0;
-      int fb = 0, fe = 0;
-      if (e < a1) {
-        const int k = Acol[e];
-        a = Aval[e];
-        fb = Brp[k];
-        fe = Brp[k + 1];
-      }
-      const int ne = min(32, a1 - e0);
-      for (int t = 0; t < ne; ++t) {
-        const double at = __shfl_sync(0xffffffffu, a, t);
-        const int f0 = __shfl_sync(0xffffffffu, fb, t);
-        const int f1 = __shfl_sync(0xffffffffu, fe, t);
-        for (int f = f0 + lane; f < f1; f += 32) {
-          const int j = Bcol[f];
-          const double prod = __dmul_rn(at, Bval[f]);
-          unsigned h = ((unsigned)j * 0x9E3779B1u) >> (32 - bits);
-          for (int probe = 0; probe < cap; ++probe) {
-            const int prev = atomicCAS(&hkey[h], -1, j);
-            if (prev == -1 || prev == j) {
-              hval[h] = __dadd_rn(hval[h], prod);
-              break;
-            }
-            h = (h + 1) & (unsigned)(cap - 1);
-          }
-        }
-        __syncwarp();
-      }
-    }
-  }
-  // 2. compact the occupied slots as (column << 32 | slot) keys
-  int d = 0;
-  for (int q0 = 0; q0 < cap; q0 += 32) {
-    const int q = q0 + lane;
-    const int c = hkey[q];
-    const unsigned m = __ballot_sync(0xffffffffu, c >= 0);
-    if (c >= 0)
-      skey[d + __popc(m & below)] = ((unsigned long long)(unsigned)c << 32) | (unsigned)q;
-    d += __popc(m);
-  }
-  int P = 1;
-  while (P < d) P <<= 1;
-  for (int q = d + lane; q < P; q += 32) skey[q] = ~0ull;
-  __syncwarp();
-  // 3. bitonic sort of the keys (ascending)
-  for (int size = 2; size <= P; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int t = lane; t < (P >> 1); t += 32) {
-        const int lo = 2 * stride * (t / stride) + (t % stride);
-        const int hi = lo + stride;
-        const bool up = (lo & size) == 0;
-        const unsigned long long x = skey[lo], y = skey[hi];
-        if ((x > y) == up) {
-          skey[lo] = y;
-          skey[hi] = x;
-        }
-      }
-      __syncwarp();
-    }
-  }
-  // 4. columns in ascending order with their sums
-  for (int r = lane; r < d; r += 32) {
-    const unsigned long long kk = skey[r];
-    cc[r] = (int)(kk >> 32);
-    cv[r] = hval[(unsigned)(kk & 0xffffffffu)];
-  }
-  if (lane == 0) cnt[i] = d;
-}
-
-// rows listed for the warp kernel: tables of CAP slots, WARPS warps per block
-// (static shared memory: 20 CAP bytes per warp); rows [first, first + count)
-// of the list, count read from the device, in list order
-template <int CAP, int WARPS>
-__global__ void __launch_bounds__(32 * WARPS) k_spgemm_rows_warp(
-    int n, const int* __restrict__ Arp, const int* __restrict__ Acol,
-    const double* __restrict__ Aval, const int* __restrict__ Brp, const int* __restrict__ Bcol,
-    const double* __restrict__ Bval, const int* __restrict__ off, const int* __restrict__ ub,
-    const int* __restrict__ wlist, const int* __restrict__ counts, int which,
-    int* __restrict__ ccol, double* __restrict__ cval, int* __restrict__ cnt) {
-  __shared__ int s_hkey[WARPS][CAP];
-  __shared__ double s_hval[WARPS][CAP];
-  __shared__ unsigned long long s_skey[WARPS][CAP];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // list 0 fills wlist from the front, list 2 from the back
-  const int count = counts[which];
-  for (int t = blockIdx.x * WARPS + w; t < count; t += gridDim.x * WARPS) {
-    const int i = which == 0 ? wlist[t] : wlist[n - 1 - t];
-    const int ex = ub[i];
-    spgemm_row_hash(i, ex, lane, CAP, Arp, Acol, Aval, Brp, Bcol, Bval, s_hkey[w], s_hval[w],
-                    s_skey[w], ccol + off[i], cval + off[i], cnt);
-    __syncwarp();
-  }
-}
-
-// rows with ex >= kSpCap: one 512-thread block per row (one block per SM)
-// with kSpBig products in dynamic shared memory. Every warp stages the
-// products of its share of row i of A (lanes over the row of B, coalesced)
-// at their canonical sequence positions; a block bitonic sort orders the
-// (column, position) keys; a block scan lists the column runs, and one
-// thread per run adds it up in sequence order. Rows beyond kSpBig are summed
-// serially.
-constexpr int kSpBig = 8192;
-constexpr int kSpBigThreads = 512;
-constexpr int kSpBigWarps = kSpBigThreads / 32;
-constexpr size_t kSpBigSmem =
-    (size_t)kSpBig * (sizeof(unsigned long long) + sizeof(double)) + (kSpBig + 1) * sizeof(int);
-
-// exclusive scan of x over the block; *total = the block's sum. s_w holds
-// kSpBigWarps + 1 ints; the block must not touch it between calls without a
-// barrier (the function ends with one).
-__device__ __forceinline__ int block_scan_excl(int x, int* s_w, int* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int incl = x;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) s_w[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    const int v = lane < kSpBigWarps ? s_w[lane] : 0;
-    int iv = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, iv, o);
-      if (lane >= o) iv += y;
-    }
-    if (lane < kSpBigWarps) s_w[lane] = iv - v;
-    if (lane == 31) s_w[kSpBigWarps] = iv;
-  }
-  __syncthreads();
-  const int r = s_w[warp] + incl - x;
-  *total = s_w[kSpBigWarps];
-  __syncthreads();
-  return r;
-}
-
-__global__ void __launch_bounds__(kSpBigThreads) k_spgemm_rows_big(
-    int n, const int* __restrict__ Arp, const int* __restrict__ Acol,
-    const double* __restrict__ Aval, const int* __restrict__ Brp, const int* __restrict__ Bcol,
-    const double* __restrict__ Bval, const int* __restrict__ off, const int* __restrict__ ub,
-    const int* __restrict__ blist, const int* __restrict__ counts,
-    int* __restrict__ ccol, double* __restrict__ cval, int* __restrict__ cnt) {
-  extern __shared__ unsigned long long s_big[];
-  unsigned long long* key = s_big;
-  double* val = reinterpret_cast<double*>(s_big + kSpBig);
-  int* start = reinterpret_cast<int*>(val + kSpBig);
-  __shared__ int s_w[kSpBigWarps + 1];
-  __shared__ int s_ak[kSpBigThreads], s_aoff[kSpBigThreads];
-  __shared__ double s_aa[kSpBigThreads];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int count = counts[1];
-  for (int t = blockIdx.x; t < count; t += gridDim.x) {
-    const int i = blist[t];
-    const int ex = ub[i];  // uniform over the block
-    int* cc = ccol + off[i];
-    double* cv = cval + off[i];
-    if (ex > kSpBig) {
-      if (tid == 0) spgemm_row_serial(i, Arp, Acol, Aval, Brp, Bcol, Bval, cc, cv, cnt);
-      __syncthreads();
-      continue;
-    }
-    // 1. products at their canonical positions (entry e of row i of A, then
-    // the row of B in order), kSpBigThreads entries of A at a time
-    const int a0 = Arp[i], a1 = Arp[i + 1];
-    int base = 0;
-    for (int c0 = a0; c0 < a1; c0 += kSpBigThreads) {
-      const int e = c0 + tid;
-      int k = 0, len = 0;
-      double a = 0.0;
-      if (e < a1) {
-        k = Acol[e];
-        a = Aval[e];
-        len = Brp[k + 1] - Brp[k];
-      }
-      int total = 0;
-      const int ex_off = block_scan_excl(len, s_w, &total);
-      s_ak[tid] = k;
-      s_aa[tid] = a;
-      s_aoff[tid] = base + ex_off;
-      __syncthreads();
-      const int nc = min(kSpBigThreads, a1 - c0);
-      for (int q = warp; q < nc; q += kSpBigWarps) {
-        const int kk = s_ak[q];
-        const double aq = s_aa[q];
-        const int fb = Brp[kk], fe = Brp[kk + 1];
-        const int pb = s_aoff[q] - fb;
-        for (int f = fb + lane; f < fe; f += 32) {
-          const int pidx = pb + f;
-          key[pidx] = ((unsigned long long)(unsigned)Bcol[f] << 32) | (unsigned)pidx;
-          val[pidx] = __dmul_rn(aq, Bval[f]);
-        }
-      }
-      base += total;
-      __syncthreads();
-    }
-    int P = 1;
-    while (P < ex) P <<= 1;
-    for (int q = ex + tid; q < P; q += kSpBigThreads) key[q] = ~0ull;
-    __syncthreads();
-    // 2. block bitonic sort
-    for (int size = 2; size <= P; size <<= 1) {
-      for (int stride = size >> 1; stride > 0; stride >>= 1) {
-        for (int u = tid; u < (P >> 1); u += kSpBigThreads) {
-          const int lo = 2 * stride * (u / stride) + (u % stride);
-          const int hi = lo + stride;
-          const bool up = (lo & size) == 0;
-          const unsigned long long x = key[lo], y = key[hi];
-          if ((x > y) == up) {
-            key[lo] = y;
-            key[hi] = x;
-          }
-        }
-        __syncthreads();
-      }
-    }
-    // 3. the start of every column run
-    int nrun = 0;
-    for (int q0 = 0; q0 < ex; q0 += kSpBigThreads) {
-      const int q = q0 + tid;
-      int st = 0;
-      if (q < ex) st = (q == 0) || ((key[q] >> 32) != (key[q - 1] >> 32));
-      int total = 0;
-      const int r = block_scan_excl(st, s_w, &total);
-      if (st) start[nrun + r] = q;
-      nrun += total;
-    }
-    if (tid == 0) start[nrun] = ex;
-    __syncthreads();
-    // 4. one thread per run, summed in sequence order
-    for (int r = tid; r < nrun; r += kSpBigThreads) {
-      const int q0 = start[r], q1 = start[r + 1];
-      double sum = 0.0;
-      for (int q = q0; q < q1; ++q) sum = __dadd_rn(sum, val[(unsigned)(key[q] & 0xffffffffu)]);
-      cc[r] = (int)(key[q0] >> 32);
-      cv[r] = sum;
-    }
-    if (tid == 0) cnt[i] = nrun;
-    __syncthreads();
-  }
-}
-
-// numeric-only C = A B on a known pattern (same canonical order)
-__global__ void k_spgemm_numeric(int n, const int* __restrict__ Arp, const int* __restrict__ Acol,
-                                 const double* __restrict__ Aval, const int* __restrict__ Brp,
-                                 const int* __restrict__ Bcol, const double* __restrict__ Bval,
-                                 const int* __restrict__ Crp, const int* __restrict__ Ccol,
-                                 double* __restrict__ Cval) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int c0 = Crp[i], c1 = Crp[i + 1];
-  for (int q = c0; q < c1; ++q) Cval[q] = 0.0;
-  for (int e = Arp[i]; e < Arp[i + 1]; ++e) {
-    const int k = Acol[e];
-    const double a = Aval[e];
-    for (int f = Brp[k]; f < Brp[k + 1]; ++f) {
-      const int q = find_in(Ccol, c0, c1, Bcol[f]);
-      Cval[q] = __dadd_rn(Cval[q], __dmul_rn(a, Bval[f]));
-    }
-  }
-}
-
-// rows of C from their slots at off[i] to the compact CSR: L lanes per row
-// (about two entries per lane on average), so that a warp's copies are a
-// few contiguous runs rather than 32 scattered rows
-template <int L>
-__global__ void k_spgemm_compact(int n, const int* __restrict__ off,
-                                 const int* __restrict__ ccol, const double* __restrict__ cval,
-                                 const int* __restrict__ Crp, int* __restrict__ Ccol,
-                                 double* __restrict__ Cval) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = (int)(t / L), lane = (int)(t % L);
-  if (i >= n) return;
-  const int o = off[i], c0 = Crp[i], len = Crp[i + 1] - c0;
-  for (int e = lane; e < len; e += L) {
-    Ccol[c0 + e] = ccol[o + e];
-    Cval[c0 + e] = cval[o + e];
-  }
-}
-
 // ------------------------------------------------------------ smoother scaling
 // l1-Jacobi scaling d_i = sign(a_ii) (|a_ii| + sum_{j != i} |a_ij|): coarse
 // Galerkin operators of the advective S~_T can have a few negative diagonals
@@ -1948,103 +1325,6 @@ int read_int(const int* d, cudaStream_t s) {
   return h;
 }
 
-// C = A B with the canonical summation order; C arrays allocated from `pool`.
-DevCSR spgemm(const DevCSR& A, const DevCSR& B, Pool& pool, Pool& scratch, cudaStream_t s) {
-  const int n = A.n;
-  int* ub = scratch.alloc<int>(n + 1);
-  int* off = scratch.alloc<int>(n + 1);
-  int* wlist = scratch.alloc<int>(n + 1);
-  int* blist = scratch.alloc<int>(n + 1);
-  int* counts = scratch.alloc<int>(3);
-  TP_CUDA_TRY(cudaMemsetAsync(counts, 0, 3 * sizeof(int), s));
-  k_spgemm_ub<<<grid_for(n), kBlock, 0, s>>>(n, A.rowptr, A.col, B.rowptr, ub, wlist, blist,
-                                             counts);
-  TP_LAUNCH_CHECK();
-  long long tot = scan_exclusive(ub, off, n, scratch, s);
-  int* ccol = scratch.alloc<int>(tot + 1);
-  double* cval = scratch.alloc<double>(tot + 1);
-  int* cnt = scratch.alloc<int>(n + 1);
-  const bool dense = B.m <= kDenseCap;
-  if (dense) {
-    static const bool dense_attr = []() {
-      TP_CUDA_TRY(cudaFuncSetAttribute(k_spgemm_dense, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kDenseSmem));
-      return true;
-    }();
-    (void)dense_attr;
-    long long blocks = ((long long)n + kDenseWarps - 1) / kDenseWarps;
-    if (blocks > 8LL * setup_sms()) blocks = 8LL * setup_sms();
-    const size_t smem = (size_t)kDenseWarps * B.m * (sizeof(double) + 1);
-    k_spgemm_dense<<<(int)blocks, 32 * kDenseWarps, smem, s>>>(
-        n, B.m, A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, off, ccol, cval, cnt);
-    TP_LAUNCH_CHECK();
-  } else {
-  k_spgemm_rows_merge<<<grid_for(n, 128), 128, 0, s>>>(n, A.rowptr, A.col, A.val, B.rowptr,
-                                                       B.col, B.val, off, ub, ccol, cval, cnt);
-  TP_LAUNCH_CHECK();
-  k_spgemm_rows<<<grid_for(n, 128), 128, 0, s>>>(n, A.rowptr, A.col, A.val, B.rowptr, B.col,
-                                                 B.val, off, ub, ccol, cval, cnt);
-  TP_LAUNCH_CHECK();
-  // SM count and the big-row kernel's shared-memory opt-in, once per process
-  // (thread-safe static initialisation; hierarchies are set up concurrently)
-  static const int num_sms = []() {
-    int dev = 0, v = 0;
-    TP_CUDA_TRY(cudaGetDevice(&dev));
-    TP_CUDA_TRY(cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev));
-    return v;
-  }();
-  {
-    // rows with kSpShort < ub < kSpMid (4 warps x 10 KiB per block), then
-    // kSpMid <= ub < kSpCap (2 warps x 20 KiB)
-    long long blocks = (n + 3) / 4;
-    if (blocks > 12LL * num_sms) blocks = 12LL * num_sms;
-    k_spgemm_rows_warp<kSpMid, 4><<<(int)blocks, 128, 0, s>>>(
-        n, A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, off, ub, wlist, counts, 0, ccol, cval,
-        cnt);
-    TP_LAUNCH_CHECK();
-    blocks = (n + 1) / 2;
-    if (blocks > 8LL * num_sms) blocks = 8LL * num_sms;
-    k_spgemm_rows_warp<kSpCap, 2><<<(int)blocks, 64, 0, s>>>(
-        n, A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, off, ub, wlist, counts, 2, ccol, cval,
-        cnt);
-  }
-  TP_LAUNCH_CHECK();
-  static const bool big_attr = []() {
-    TP_CUDA_TRY(cudaFuncSetAttribute(k_spgemm_rows_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kSpBigSmem));
-    return true;
-  }();
-  (void)big_attr;
-  k_spgemm_rows_big<<<n < num_sms ? n : num_sms, kSpBigThreads, kSpBigSmem, s>>>(
-      n, A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, off, ub, blist, counts, ccol, cval, cnt);
-  TP_LAUNCH_CHECK();
-  }
-  DevCSR C;
-  C.n = n;
-  C.m = B.m;
-  C.rowptr = pool.alloc<int>(n + 1);
-  long long nnz = scan_exclusive(cnt, C.rowptr, n, scratch, s);
-  C.nnz = (int)nnz;
-  C.col = pool.alloc<int>(nnz + 1);
-  C.val = pool.alloc<double>(nnz + 1);
-  {
-    const double avg = n > 0 ? (double)nnz / n : 1.0;
-    int L = 1;
-    while (L < 32 && 2.0 * L < avg) L *= 2;
-    const int g = grid_for((long long)n * L);
-    switch (L) {
-#define TP_CASE(LL)                                                                          \
-  case LL:                                                                                   \
-    k_spgemm_compact<LL><<<g, kBlock, 0, s>>>(n, off, ccol, cval, C.rowptr, C.col, C.val); \
-    break;
-      TP_CASE(1) TP_CASE(2) TP_CASE(4) TP_CASE(8) TP_CASE(16) TP_CASE(32)
-#undef TP_CASE
-    }
-  }
-  TP_LAUNCH_CHECK();
-  return C;
-}
-
 DevCSR transpose(const DevCSR& P, Pool& pool, Pool& scratch, cudaStream_t s) {
   DevCSR R;
   R.n = P.m;
@@ -2075,17 +1355,6 @@ DevCSR transpose(const DevCSR& P, Pool& pool, Pool& scratch, cudaStream_t s) {
 }
 
 }  // namespace
-
-DevCSR csr_product(const DevCSR& A, const DevCSR& B, Pool& pool, Pool& scratch,
-                   cudaStream_t s) {
-  return spgemm(A, B, pool, scratch, s);
-}
-
-void csr_product_numeric(const DevCSR& A, const DevCSR& B, const DevCSR& C, cudaStream_t s) {
-  k_spgemm_numeric<<<grid_for(A.n, 128), 128, 0, s>>>(A.n, A.rowptr, A.col, A.val, B.rowptr,
-                                                      B.col, B.val, C.rowptr, C.col, C.val);
-  TP_LAUNCH_CHECK();
-}
 
 void csr_transpose_positions(const DevCSR& A, int* tpos, int* err, cudaStream_t s) {
   if (A.n > 0 && A.nnz >= (long long)kWarpRowMean * A.n)
@@ -2297,8 +1566,8 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
     phase_ms[1] += clk.lap(s);
     cur.R = transpose(P, pool, scratch, s);
     phase_ms[2] += clk.lap(s);
-    cur.AP = spgemm(A, P, pool, scratch, s);
-    DevCSR Ac = spgemm(cur.R, cur.AP, pool, scratch, s);
+    cur.AP = csr_product(A, P, pool, scratch, s);
+    DevCSR Ac = csr_product(cur.R, cur.AP, pool, scratch, s);
     TP_CUDA_TRY(cudaStreamSynchronize(s));
     phase_ms[3] += clk.lap(s);
     scratch.release();
@@ -2531,16 +1800,10 @@ void Hierarchy::refresh(cudaStream_t s) {
   if (L.empty()) fail(TP_ESTATE, "AMG: refresh before setup");
   for (size_t l = 0; l + 1 < L.size(); ++l) {
     Level& v = L[l];
-    const int n = v.A.n;
-    k_spgemm_numeric<<<grid_for(n, 128), 128, 0, s>>>(n, v.A.rowptr, v.A.col, v.A.val,
-                                                      v.P.rowptr, v.P.col, v.P.val, v.AP.rowptr,
-                                                      v.AP.col, v.AP.val);
-    TP_LAUNCH_CHECK();
+    csr_product_numeric(v.A, v.P, v.AP, scratch, s);
     Level& c = L[l + 1];
-    k_spgemm_numeric<<<grid_for(c.A.n, 128), 128, 0, s>>>(c.A.n, v.R.rowptr, v.R.col, v.R.val,
-                                                          v.AP.rowptr, v.AP.col, v.AP.val,
-                                                          c.A.rowptr, c.A.col, c.A.val);
-    TP_LAUNCH_CHECK();
+    csr_product_numeric(v.R, v.AP, c.A, scratch, s);
+    scratch.release();
   }
   finish_levels(s, false);
 }

@@ -1172,7 +1172,8 @@ void schur_diag_values(tp_ctx* c, bool symbolic) {
     c->Sd = c->Cd;
     c->Sd.val = c->dpool.alloc<double>(c->Cd.nnz);
   } else {
-    csr_product_numeric(ATp, B, c->Cd, s);
+    c->dscratch.release();
+    csr_product_numeric(ATp, B, c->Cd, c->dscratch, s);
   }
   k_schur_diag_merge<<<grid_for(N), kBlock, 0, s>>>(N, c->Cd.rowptr, c->Cd.col, c->Cd.val,
                                                     c->rowptr, c->col, c->ATT, c->Sd.val);

@@ -70,3 +70,31 @@ def test_interpolation_and_galerkin_rows_are_bit_exact(n, degree, hubs, interp):
 @pytest.mark.parametrize("interp", [0, 1])
 def test_interpolation_widths_are_bit_exact(pmax, interp):
     compare(graph_matrix(600, 14, seed=pmax, positive=0.2), interp, pmax, 2)
+
+
+# rows of R (A P) with 236 columns on average and up to 505 out of 2842 (past
+# the dense-row kernel), from fewer and from more than 1024 products
+def test_products_past_the_group_kernels_are_bit_exact():
+    compare(graph_matrix(12000, 24, seed=12024, positive=0.1), 0, 4, 3)
+
+
+def test_refreshed_galerkin_values_are_the_products_of_their_factors():
+    """Newton with structure reuse refreshes the Galerkin values on known
+    patterns: every operator below the first Galerkin level equals R (A P) of
+    the level above it in the oracle's order, bit for bit (level 0's own values
+    have moved on to the next state by the time they can be read)."""
+    from synthetic import make_problem
+    prob = make_problem("tiny", shape=(40, 36, 12), seed=11, dt_days=0.5)
+    s = thermo.Solver.from_problem(prob)
+    s.newton_step(prob["p_n"], prob["T_n"], prob["dt"], max_newton=2, tol_f=0.0, tol_dx=0.0,
+                  rtol=1e-12, reuse=True)
+    for w in (0, 1):
+        n, _ = s.hierarchy_info(w)
+        assert n.size > 2
+        levels = [s.export_level(w, l) for l in range(n.size)]
+        for fine, coarse in zip(levels[1:], levels[2:]):
+            P = fine["P"]
+            C = oamg.galerkin(fine["A"], P, oamg.transpose(P, coarse["cf"].size))
+            for a, b in zip(C, coarse["A"]):
+                assert np.array_equal(a, b), w
+    s.close()
