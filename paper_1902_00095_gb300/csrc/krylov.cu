@@ -19,13 +19,16 @@ namespace tp {
 
 namespace {
 
-// vectors per multi-dot launch: 16 while the basis vectors are short (the
-// launches dominate), 4 for long ones (fewer concurrent DRAM streams).
-// FGMRES time measured on 262k / 2.1M / 8.4M unknowns: 16 vectors 34.0 /
-// 49.0 / 4988 ms, 8 vectors 34.5 / 50.2 / 5583 ms, 4 vectors 34.8 / 48.3 /
-// 4827 ms.
-constexpr int kDotWide = 16, kDotNarrow = 4;
-constexpr long long kDotWideMaxN = 1ll << 20;  // vector length up to which 16 are taken
+// vectors per multi-dot launch: 8 while the basis vectors are short (the
+// launches and the warps' reductions dominate), 4 for long ones (a thread's
+// loads of four elements fit its registers). Kernel time of the dots of a
+// solve: 8.4 M unknowns, 4 vectors 7.5 ms (66 % of the FP64 pipe's rate; 10.4
+// with one element at a time and five additions per value and warp), 8 vectors
+// 10.7 ms; 262 k unknowns, 8 vectors 0.86 ms, 16 vectors 1.06 ms (1.16 before).
+// The order of every sum is fixed by the grid and block sizes alone.
+constexpr int kDotWide = 8, kDotNarrow = 4;
+constexpr int kDotWideU = 2, kDotNarrowU = 4;  // elements a thread loads at a time
+constexpr long long kDotWideMaxN = 1ll << 20;  // vector length up to which 8 are taken
 constexpr int kEstSlot = 16;  // pinned-buffer offset of the two convergence-estimate slots
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -151,10 +154,34 @@ __global__ void __launch_bounds__(256) k_block_spmv(int N, const int* __restrict
 }
 
 // ------------------------------------------------------------ Gram-Schmidt
+// sums of acc[0..NV) over the warp, each with warp_sum's tree: after the call
+// the lanes with lane % (32 / NV) == 0 hold the sum of acc[lane / (32 / NV)] in
+// acc[0]. Each step exchanges half of the values a lane still holds, so the NV
+// sums take NV - 1 additions and log2(32 / NV) more, not 5 NV: an FP64 addition
+// occupies the FP64 pipe for the whole warp, and five per value kept it busy
+// for longer than the products of a short vector.
+template <int NV>
+__device__ __forceinline__ void warp_sums(double (&acc)[NV]) {
+  const int lane = threadIdx.x & 31;
+  int o = 16;
+#pragma unroll
+  for (int c = NV / 2; c > 0; c >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int q = 0; q < c; ++q) {
+      const double give = up ? acc[q] : acc[q + c];
+      const double keep = up ? acc[q + c] : acc[q];
+      acc[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+}
+
 // partial dot products V_k . w, k0 <= k < k0 + nv (nv <= NV), of this
 // block's element chunk: per-thread sums, then warp sums, then the block's
 // warps in order (one barrier)
-template <int NV>
+template <int NV, int U>
 __global__ void __launch_bounds__(256) k_mdot(long long n2, const double* __restrict__ V,
                                               long long stride, int k0, int nv,
                                               const double* __restrict__ w,
@@ -169,20 +196,35 @@ __global__ void __launch_bounds__(256) k_mdot(long long n2, const double* __rest
   double acc[NV];
 #pragma unroll
   for (int q = 0; q < NV; ++q) acc[q] = 0.0;
-  for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+  const double* Vk = V + (long long)k0 * stride;
+  long long i = lo + threadIdx.x;
+  // the loads of U elements in flight; each thread's sums stay in element order
+  const int bd = blockDim.x;
+  for (; i + (U - 1) * bd < hi; i += U * bd) {
+    double wu[U], v[U][NV];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      wu[u] = w[i + u * bd];
+#pragma unroll
+      for (int q = 0; q < NV; ++q)
+        if (q < nv) v[u][q] = Vk[q * stride + i + u * bd];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int q = 0; q < NV; ++q)
+        if (q < nv) acc[q] = fma(wu[u], v[u][q], acc[q]);
+  }
+  for (; i < hi; i += bd) {
     const double wi = w[i];
 #pragma unroll
     for (int q = 0; q < NV; ++q)
-      if (q < nv) acc[q] += wi * V[(long long)(k0 + q) * stride + i];
+      if (q < nv) acc[q] = fma(wi, Vk[q * stride + i], acc[q]);
   }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < NV; ++q) {
-    if (q < nv) {
-      const double t = warp_sum(acc[q]);
-      if (lane == 0) sh[wid][q] = t;
-    }
-  }
+  warp_sums<NV>(acc);
+  constexpr int kPer = 32 / NV;
+  if (lane % kPer == 0) sh[wid][lane / kPer] = acc[0];
   __syncthreads();
   if (threadIdx.x < nv) {
     double t = 0.0;
@@ -440,9 +482,9 @@ void mdot_all(long long n2, const double* V, long long stride, int count, const 
   for (int k0 = 0; k0 < count; k0 += nvmax) {
     const int nv = count - k0 < nvmax ? count - k0 : nvmax;
     if (nvmax == kDotWide)
-      launch_pdl(k_mdot<kDotWide>, B, 256, s, n2, V, stride, k0, nv, w, partials, gate);
+      launch_pdl(k_mdot<kDotWide, kDotWideU>, B, 256, s, n2, V, stride, k0, nv, w, partials, gate);
     else
-      launch_pdl(k_mdot<kDotNarrow>, B, 256, s, n2, V, stride, k0, nv, w, partials, gate);
+      launch_pdl(k_mdot<kDotNarrow, kDotNarrowU>, B, 256, s, n2, V, stride, k0, nv, w, partials, gate);
   }
   launch_pdl(k_reduce_rows, count, 256, s, count, B, partials, out, gate);
 }
