@@ -598,7 +598,7 @@ int tp_export_system(tp_ctx* c, int* rowptr, int* col, double* val, double* schu
     TP_CUDA_TRY(cudaMemcpyAsync(schur_val, c->Sval, c->nnzb * sizeof(double), cudaMemcpyDeviceToHost, s));
   if (scales) {
     if (!c->built) {
-      tp::launch_extract_blocks(c->nnzb, c->bval, c->App, c->ApT, c->ATp, c->ATT, s);
+      tp::extract_blocks(c);
       tp::launch_equation_scales(c->N, c->dpos, c->App, c->ATT, c->tmpN, c->partials, c->nparts,
                                  c->scales, s);
     }
@@ -1095,6 +1095,18 @@ int assemble_device(tp_ctx* c, double dt) {
   return TP_OK;
 }
 
+// the scalar blocks of the assembled matrix on its pattern, and the coupling
+// blocks by grid direction
+void extract_blocks(tp_ctx* c) {
+  launch_extract_blocks(c->nnzb, c->bval, c->App, c->ApT, c->ATp, c->ATT, c->s);
+  if (c->grid.nx < 2 || c->grid.ny < 2 || c->grid.nz < 2) return;
+  if (!c->ApT_grid) {
+    c->ApT_grid = c->pool.alloc<double>(7 * (size_t)c->N);
+    c->ATp_grid = c->pool.alloc<double>(7 * (size_t)c->N);
+  }
+  launch_coupling_planes(c->grid, c->rowptr, c->bval, c->ApT_grid, c->ATp_grid, c->s);
+}
+
 // features -> MLP -> corrected S~ with the per-row guard; more than a quarter
 // of the rows falling back switches the whole matrix back to plain S~
 void learned_features(tp_ctx* c) {
@@ -1105,7 +1117,7 @@ void learned_features(tp_ctx* c) {
     c->S_learned = c->lpool.alloc<double>(c->nnzb);
     c->nbad = c->lpool.alloc<int>(1);
   }
-  launch_extract_blocks(c->nnzb, c->bval, c->App, c->ApT, c->ATp, c->ATT, s);
+  extract_blocks(c);
   launch_equation_scales(c->N, c->dpos, c->App, c->ATT, c->tmpN, c->partials, c->nparts,
                          c->scales, s);
   launch_features(c->grid, c->fluid, c->dpos, c->Tf3, c->Tc3, c->phi, c->p, c->T,
@@ -1193,7 +1205,7 @@ void build_device(tp_ctx* c, const tp_precond_opts& o) {
   c->probe_nodes.clear();
   c->probe_set = 0;
   c->built = false;
-  launch_extract_blocks(c->nnzb, c->bval, c->App, c->ApT, c->ATp, c->ATT, s);
+  extract_blocks(c);
   launch_equation_scales(c->N, c->dpos, c->App, c->ATT, c->tmpN, c->partials, c->nparts,
                          c->scales, s);
   c->S_active = (o.schur == 2) ? c->ATT : c->Sval;
@@ -1320,7 +1332,7 @@ void build_device(tp_ctx* c, const tp_precond_opts& o) {
 void refresh_device(tp_ctx* c) {
   cudaStream_t s = c->s;
   // A_pp and (for schur = 2) A_TT planes are the level-0 values in place
-  launch_extract_blocks(c->nnzb, c->bval, c->App, c->ApT, c->ATp, c->ATT, s);
+  extract_blocks(c);
   if (c->opts.schur == 1) {
     learned_schur_values(c);
     if (c->learned_global_fallback)

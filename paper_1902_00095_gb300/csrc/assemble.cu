@@ -333,6 +333,28 @@ __global__ void k_extract(int nnzb, const double4_32a* __restrict__ bval, double
   ATT[e] = b.w;
 }
 
+__global__ void k_coupling_planes(GridDev g, const int* __restrict__ rowptr,
+                                  const double4_32a* __restrict__ bval,
+                                  double* __restrict__ ApT, double* __restrict__ ATp) {
+  const int N = g.nx * g.ny * g.nz;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  const int x = i % g.nx, y = (i / g.nx) % g.ny, z = i / (g.nx * g.ny);
+  const bool has[7] = {z > 0, y > 0, x > 0, true, x < g.nx - 1, y < g.ny - 1, z < g.nz - 1};
+  int e = rowptr[i];
+#pragma unroll
+  for (int k = 0; k < 7; ++k) {
+    double pt = 0.0, tp = 0.0;
+    if (has[k]) {
+      const double4_32a b = bval[e++];
+      pt = b.y;
+      tp = b.z;
+    }
+    ApT[(long long)k * N + i] = pt;
+    ATp[(long long)k * N + i] = tp;
+  }
+}
+
 __global__ void k_abs_diag(int N, const int* __restrict__ dpos, const double* __restrict__ A,
                            double* __restrict__ out) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -465,6 +487,13 @@ void launch_extract_blocks(int nnzb, const double* bval, double* App, double* Ap
                            double* ATT, cudaStream_t s) {
   k_extract<<<grid_for(nnzb), kBlock, 0, s>>>(nnzb, reinterpret_cast<const double4_32a*>(bval), App,
                                               ApT, ATp, ATT);
+  TP_LAUNCH_CHECK();
+}
+
+void launch_coupling_planes(const GridDev& g, const int* rowptr, const double* bval,
+                            double* ApT_grid, double* ATp_grid, cudaStream_t s) {
+  k_coupling_planes<<<grid_for(g.nx * g.ny * g.nz), kBlock, 0, s>>>(
+      g, rowptr, reinterpret_cast<const double4_32a*>(bval), ApT_grid, ATp_grid);
   TP_LAUNCH_CHECK();
 }
 

@@ -50,6 +50,11 @@ void launch_wells(const GridDev& g, const FluidDev& f, const WellsDev& w, const 
                   double* bval, double* Sval, double* Rm, double* Re, cudaStream_t s);
 void launch_extract_blocks(int nnzb, const double* bval, double* App, double* ApT, double* ATp,
                            double* ATT, cudaStream_t s);
+// The off-diagonal blocks by grid direction: plane k of A_pT (A_Tp) holds row
+// i's entry at column i + (-nxy, -nx, -1, 0, +1, +nx, +nxy)[k], 0 where the
+// grid has no such neighbour ([7][N]; every grid extent at least 2).
+void launch_coupling_planes(const GridDev& g, const int* rowptr, const double* bval,
+                            double* ApT_grid, double* ATp_grid, cudaStream_t s);
 // s_m = N / sum |A_pp,ii|, s_e = N / sum |A_TT,ii| into scales[0..1].
 void launch_equation_scales(int N, const int* dpos, const double* App, const double* ATT,
                             double* tmp, double* partials, int nparts, double* scales,

@@ -97,6 +97,40 @@ __global__ void k_rhs_minus(int N, const int* __restrict__ rp, const int* __rest
   out[i] = bi - acc;
 }
 
+// the same with the plane stored by grid direction (launch_coupling_planes):
+// coalesced loads, no column indices, the row's values loaded before the
+// dependency wait (the planes do not change during a solve). An absent
+// neighbour's value is 0 and its column is the row's own; the sum runs in the
+// CSR row's order. Bound by HBM (80 bytes per row, 50 us at 4.2 M rows); from
+// the CSR plane, one thread per row striding over its entries, it took 76 us
+// after the V-cycle before it ended. The layered 256x256x64 solve (two per
+// iteration) 113.7 -> 112.9 ms.
+__global__ void __launch_bounds__(256) k_rhs_minus_grid(int N, int nx, int nxy,
+                                                        const double* __restrict__ plane,
+                                                        const double* __restrict__ b,
+                                                        const double* __restrict__ x,
+                                                        double* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  double v[7];
+#pragma unroll
+  for (int k = 0; k < 7; ++k) v[k] = i < N ? plane[(long long)k * N + i] : 0.0;
+  pdl_wait();
+  pdl_trigger();
+  if (i >= N) return;
+  const double bi = b[i];
+  const int o[7] = {-nxy, -nx, -1, 0, 1, nx, nxy};
+  double xv[7];
+#pragma unroll
+  for (int k = 0; k < 7; ++k) {
+    const int j = i + o[k];
+    xv[k] = x[j >= 0 && j < N ? j : i];
+  }
+  double acc = 0.0;
+#pragma unroll
+  for (int k = 0; k < 7; ++k) acc += v[k] * xv[k];
+  out[i] = bi - acc;
+}
+
 // w = D A z (block-CSR, Eq. AXR); optionally stores z into Z_j.
 __global__ void __launch_bounds__(256) k_block_spmv(int N, const int* __restrict__ rp,
                                                     const int* __restrict__ col,
@@ -724,18 +758,27 @@ void launch_block_spmv(int N, const int* rowptr, const int* col, const double* b
   TP_LAUNCH_CHECK();
 }
 
+// out = b - A x for a coupling block: from its planes by grid direction when
+// the context keeps them (every grid extent at least 2), else from CSR
+static void rhs_minus(tp_ctx* c, const double* csr, const double* plane, const double* b,
+                      const double* x, double* out, cudaStream_t s) {
+  const int N = c->N;
+  if (plane)
+    launch_pdl(k_rhs_minus_grid, grid_for(N), kBlock, s, N, c->grid.nx, c->grid.nx * c->grid.ny,
+               plane, b, x, out);
+  else
+    launch_pdl(k_rhs_minus, grid_for(N), kBlock, s, N, c->rowptr, c->col, csr, b, x, out);
+}
+
 void precond_record(tp_ctx* c, cudaStream_t s) {
   c->probe.npairs = 0;
   Hierarchy& hp = *c->hpp;
   Hierarchy& hs = *c->hS;
-  const int N = c->N;
   hp.vcycle(s);  // step 1: x_p = V_pp(b_p)
-  launch_pdl(k_rhs_minus, grid_for(N), kBlock, s, N, c->rowptr, c->col, c->ATp, c->bT_s, hp.out,
-             hs.in);  // step 2
+  rhs_minus(c, c->ATp, c->ATp_grid, c->bT_s, hp.out, hs.in, s);  // step 2
   hs.vcycle(s);  // step 3: d_T = V_S(bt_T)
   if (c->opts.variant == 0) {
-    launch_pdl(k_rhs_minus, grid_for(N), kBlock, s, N, c->rowptr, c->col, c->ApT, c->bp_s,
-               hs.out, hp.in);  // step 4
+    rhs_minus(c, c->ApT, c->ApT_grid, c->bp_s, hs.out, hp.in, s);  // step 4
     hp.vcycle(s);  // step 5: d_p = V_pp(bt_p)
   }
 }

@@ -93,7 +93,7 @@ int newton_step(tp_ctx* c, double dt, const tp_precond_opts& popts, const tp_new
   // linearise at x_0
   int st = assemble_device(c, dt);
   if (st != TP_OK) return st;
-  launch_extract_blocks(c->nnzb, c->bval, c->App, c->ApT, c->ATp, c->ATT, s);
+  extract_blocks(c);
   launch_equation_scales(N, c->dpos, c->App, c->ATT, c->tmpN, c->partials, c->nparts,
                          c->scales, s);
   // the first linearisation fixes the scaling of the function norm
@@ -136,7 +136,7 @@ int newton_step(tp_ctx* c, double dt, const tp_precond_opts& popts, const tp_new
       if (st != TP_OK && st != TP_ENONFINITE) return st;
       const bool finite = st == TP_OK;
       if (finite) {
-        launch_extract_blocks(c->nnzb, c->bval, c->App, c->ApT, c->ATp, c->ATT, s);
+        extract_blocks(c);
         launch_equation_scales(N, c->dpos, c->App, c->ATT, c->tmpN, c->partials, c->nparts,
                                c->scales, s);
         Gt = std::sqrt(sumsq2(c, c->Rm, c->Re, c->fscale));

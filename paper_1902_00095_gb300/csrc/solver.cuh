@@ -33,6 +33,9 @@ struct tp_ctx {
   double* Sval = nullptr;  // [nnzb]
   double *Rm = nullptr, *Re = nullptr;
   double *App = nullptr, *ApT = nullptr, *ATp = nullptr, *ATT = nullptr;
+  // A_pT and A_Tp by grid direction ([7][N], k_coupling_planes), null when a
+  // grid extent is 1
+  double *ApT_grid = nullptr, *ATp_grid = nullptr;
   double* scales = nullptr;  // [2] equation scales s_m, s_e
   double* ones = nullptr;    // [2] = {1, 1}
   double* fscale = nullptr;  // [2] scaling of the Newton function norm
@@ -100,6 +103,7 @@ int fgmres_solve(tp_ctx* c, const double* bp, const double* bT, double* xp, doub
                  double rtol, int maxit, int restart, tp_solve_info* info);
 // device-resident steps shared by the C-ABI calls and the Newton driver
 int assemble_device(tp_ctx* c, double dt);              // at (c->p, c->T)
+void extract_blocks(tp_ctx* c);                          // the blocks of c->bval
 void build_device(tp_ctx* c, const tp_precond_opts& o);  // full setup + graph
 void refresh_device(tp_ctx* c);                          // numeric-only
 void negated_residual(tp_ctx* c);                        // io0, io1 = -G

