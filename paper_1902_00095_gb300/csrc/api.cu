@@ -53,9 +53,12 @@ __global__ void k_check_fields(int N, const double* Kx, const double* Ky, const 
     atomicOr(flags, 2);
 }
 
-__global__ void k_check_finite(long long n, const double* a, int* flags) {
+__global__ void k_check_state(long long n, const double* a, const double* b, const double* c,
+                              const double* d, int* flags) {
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i < n && !isfinite(a[i])) atomicOr(flags, 1);
+  if (i >= n) return;
+  if (!isfinite(a[i]) || !isfinite(b[i]) || !isfinite(c[i]) || !isfinite(d[i]))
+    atomicOr(flags, 1);
 }
 
 __global__ void k_negate(double* a, long long n) {
@@ -1075,20 +1078,15 @@ int assemble_device(tp_ctx* c, double dt) {
   const long long n = c->N;
   int* flags = reinterpret_cast<int*>(c->partials);
   TP_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int), s));
-  for (const double* a : {c->p, c->T, c->pn, c->Tn}) {
-    k_check_finite<<<grid_for(n), kBlock, 0, s>>>(n, a, flags);
-    TP_LAUNCH_CHECK();
-  }
+  k_check_state<<<grid_for(n), kBlock, 0, s>>>(n, c->p, c->T, c->pn, c->Tn, flags);
+  TP_LAUNCH_CHECK();
   if (read_flags(flags, s)) return TP_ENONFINITE;
   launch_cell_props(c->N, c->p, c->T, c->fluid, c->rho, c->lam, c->lam_p, c->lam_T, s);
   launch_assemble(c->grid, c->fluid, c->rowptr, c->dpos, c->Tf3, c->Tc3, c->phi, c->p, c->T,
                   c->pn, c->Tn, c->rho, c->lam, c->lam_p, c->lam_T, dt, c->bval, c->Sval, c->Rm,
-                  c->Re, s);
+                  c->Re, flags, s);
   launch_wells(c->grid, c->fluid, c->wells, c->dpos, c->Kx, c->Ky, c->p, c->T, c->rho, c->lam,
-               c->lam_p, c->lam_T, c->bval, c->Sval, c->Rm, c->Re, s);
-  TP_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int), s));
-  k_check_finite<<<grid_for(4ll * c->nnzb), kBlock, 0, s>>>(4ll * c->nnzb, c->bval, flags);
-  TP_LAUNCH_CHECK();
+               c->lam_p, c->lam_T, c->bval, c->Sval, c->Rm, c->Re, flags, s);
   if (read_flags(flags, s)) return TP_ENONFINITE;
   c->assembled = true;
   c->dt_last = dt;

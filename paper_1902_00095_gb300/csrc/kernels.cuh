@@ -38,16 +38,17 @@ void launch_cell_props(int N, const double* p, const double* T, const FluidDev& 
 // neighbour ([3][N], axis-major), from the fields.
 void launch_face_trans(const GridDev& g, const double* Kx, const double* Ky, const double* Kz,
                        const double* kT, double* Tf3, double* Tc3, cudaStream_t s);
-// Jacobian (block-CSR, 4 doubles per block), residual and S~_T values.
+// Jacobian (block-CSR, 4 doubles per block), residual and S~_T values; here and
+// in launch_wells *flags gets bit 1 when a block entry written is not finite.
 void launch_assemble(const GridDev& g, const FluidDev& f, const int* rowptr, const int* dpos,
                      const double* Tf3, const double* Tc3, const double* phi, const double* p,
                      const double* T, const double* p_n, const double* T_n, const double* rho,
                      const double* lam, const double* lam_p, const double* lam_T, double dt,
-                     double* bval, double* Sval, double* Rm, double* Re, cudaStream_t s);
+                     double* bval, double* Sval, double* Rm, double* Re, int* flags, cudaStream_t s);
 void launch_wells(const GridDev& g, const FluidDev& f, const WellsDev& w, const int* dpos,
                   const double* Kx, const double* Ky, const double* p, const double* T,
                   const double* rho, const double* lam, const double* lam_p, const double* lam_T,
-                  double* bval, double* Sval, double* Rm, double* Re, cudaStream_t s);
+                  double* bval, double* Sval, double* Rm, double* Re, int* flags, cudaStream_t s);
 void launch_extract_blocks(int nnzb, const double* bval, double* App, double* ApT, double* ATp,
                            double* ATT, cudaStream_t s);
 // The off-diagonal blocks by grid direction: plane k of A_pT (A_Tp) holds row
