@@ -285,7 +285,7 @@ int tp_export_system(tp_ctx* ctx, int* rowptr, int* col, double* val,
 int tp_vcycle_measure(tp_ctx* ctx, int which, int reps, double* ms, double* bytes,
                       double* opc);
 
-/* Host wall time (ms) of the last AMG setup of hierarchy which (0 A_pp,
+/* Time (ms, on its stream) of the last AMG setup of hierarchy which (0 A_pp,
  * 1 Schur) by phase: ms[0] strength + PMIS, ms[1] interpolation,
  * ms[2] transpose, ms[3] Galerkin products, ms[4] smoother scaling, ELL copy
  * and coarsest inverse. */

@@ -198,7 +198,7 @@ class Hierarchy {
   Pool pool;
   Pool scratch;   // setup temporaries (rewound after every level)
   double* coarse_dense = nullptr;   // [nc*nc] work for the inverse
-  // host wall time of the setup phases (ms): strength + PMIS, interpolation,
+  // time of the setup phases on its stream (ms): strength + PMIS, interpolation,
   // transpose, Galerkin products, smoother scaling + coarse inverse
   double phase_ms[5] = {0, 0, 0, 0, 0};
   int* err = nullptr;
@@ -210,6 +210,10 @@ class Hierarchy {
   std::vector<TailLevel> tail_host;
 
  private:
+  std::vector<cudaEvent_t> phase_ev;  // kept between setups
+  std::vector<int> marks;             // phase that ends at phase_ev[q]
+  void mark_phase(int phase, cudaStream_t s);
+  void read_phases();
   void finish_levels(cudaStream_t s, bool allocate);
   void plan_tail(cudaStream_t s);
   void vcycle_fp64(cudaStream_t s);

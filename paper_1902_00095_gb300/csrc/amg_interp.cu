@@ -549,12 +549,11 @@ bool truncated_interpolation(const DevCSR& A, bool extended, int sms, const int*
   w.ocnt = scratch.alloc<int>(3);
   if (extended) interp_tiers<true>(A, sms, dpos, strong, state, cidx, pmax, w, s);
   else interp_tiers<false>(A, sms, dpos, strong, state, cidx, pmax, w, s);
-  int over = 0;  // rows past the last capacities; read with the scan's total
-  TP_CUDA_TRY(cudaMemcpyAsync(&over, w.ocnt + 2, sizeof(int), cudaMemcpyDeviceToHost, s));
+  int over = 0;  // rows past the last capacities
   P.n = n;
   P.m = nc;
   P.rowptr = pool.alloc<int>(n + 1);
-  const long long total = scan_exclusive(w.cnt, P.rowptr, n, scratch, s);
+  const long long total = scan_exclusive(w.cnt, P.rowptr, n, scratch, s, w.ocnt + 2, &over);
   if (over > 0) return false;
   P.nnz = (int)total;
   P.col = pool.alloc<int>(P.nnz + 1);

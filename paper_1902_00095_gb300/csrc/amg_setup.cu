@@ -8,7 +8,6 @@
 // its distance-two extended+i form; all structure-deciding arithmetic uses
 // __dmul_rn / __dadd_rn / __ddiv_rn in a fixed ascending-column order.
 #include "amg_dev.cuh"
-#include <chrono>
 #include <cmath>
 #include <algorithm>
 
@@ -105,8 +104,9 @@ __global__ void k_pmis_select(int n, const int* __restrict__ rp, const int* __re
                               const unsigned char* __restrict__ strong,
                               const int* __restrict__ tpos, const int* __restrict__ lam,
                               const signed char* __restrict__ state, unsigned long long seed,
-                              unsigned char* __restrict__ newc) {
+                              unsigned char* __restrict__ newc, int* __restrict__ undecided) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) *undecided = 0;  // set again by this round's k_pmis_update
   if (i >= n) return;
   if (state[i] != kU) {
     newc[i] = 0;
@@ -149,7 +149,7 @@ __global__ void k_pmis_update(int n, const int* __restrict__ rp, const int* __re
       return;
     }
   }
-  atomicAdd(undecided, 1);
+  *undecided = 1;  // the same value from every point that is left
 }
 
 // One-warp-per-row forms of the strength and PMIS kernels above, for levels
@@ -208,9 +208,11 @@ __global__ void k_pmis_select_warp(int n, const int* __restrict__ rp,
                                    const unsigned char* __restrict__ strong,
                                    const int* __restrict__ tpos, const int* __restrict__ lam,
                                    const signed char* __restrict__ state,
-                                   unsigned long long seed, unsigned char* __restrict__ newc) {
+                                   unsigned long long seed, unsigned char* __restrict__ newc,
+                                   int* __restrict__ undecided) {
   int lane;
   const int i = warp_row(lane);
+  if (i == 0 && lane == 0) *undecided = 0;  // set again by this round's update
   if (i >= n) return;
   if (state[i] != kU) {
     if (lane == 0) newc[i] = 0;
@@ -253,13 +255,8 @@ __global__ void k_pmis_update_warp(int n, const int* __restrict__ rp,
   const bool any = __any_sync(0xffffffffu, c);
   if (lane == 0) {
     if (any) state[i] = kF;
-    else atomicAdd(undecided, 1);
+    else *undecided = 1;
   }
-}
-
-__global__ void k_cflag(int n, const signed char* __restrict__ state, int* __restrict__ flag) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) flag[i] = state[i] == kC ? 1 : 0;
 }
 
 // ---------------------------------------------------- classical interpolation
@@ -866,22 +863,23 @@ __global__ void k_trunc_fill(int n, const int* __restrict__ Prp, const int* __re
 }
 
 // ------------------------------------------------------------- transpose
+// entries per column, and every entry's place among its column's (in no
+// particular order)
 __global__ void k_count_cols(int n, const int* __restrict__ rp, const int* __restrict__ col,
-                             int* __restrict__ cnt) {
+                             int* __restrict__ cnt, int* __restrict__ place) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  for (int e = rp[i]; e < rp[i + 1]; ++e) atomicAdd(&cnt[col[e]], 1);
+  for (int e = rp[i]; e < rp[i + 1]; ++e) place[e] = atomicAdd(&cnt[col[e]], 1);
 }
 
 __global__ void k_fill_transpose(int n, const int* __restrict__ rp, const int* __restrict__ col,
                                  const double* __restrict__ val, const int* __restrict__ Trp,
-                                 int* __restrict__ cursor, int* __restrict__ Tcol,
+                                 const int* __restrict__ place, int* __restrict__ Tcol,
                                  double* __restrict__ Tval) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   for (int e = rp[i]; e < rp[i + 1]; ++e) {
-    int c = col[e];
-    int q = Trp[c] + atomicAdd(&cursor[c], 1);
+    const int q = Trp[col[e]] + place[e];
     Tcol[q] = i;
     Tval[q] = val[e];
   }
@@ -1181,12 +1179,13 @@ __global__ void k_to_stencil(int n, int nx, int nxy, const int* __restrict__ rp,
 }
 
 // ------------------------------------------------------------ coarsest level
+// the entries of a CSR matrix into a zeroed dense one, one warp per row
 __global__ void k_to_dense(int n, const int* __restrict__ rp, const int* __restrict__ col,
                            const double* __restrict__ val, double* __restrict__ D) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   if (i >= n) return;
-  for (int j = 0; j < n; ++j) D[(long long)i * n + j] = 0.0;
-  for (int e = rp[i]; e < rp[i + 1]; ++e) D[(long long)i * n + col[e]] += val[e];
+  for (int e = rp[i] + (threadIdx.x & 31); e < rp[i + 1]; e += 32)
+    D[(long long)i * n + col[e]] = 0.0 + val[e];
 }
 
 // Gauss-Jordan elimination with partial pivoting on [A | I] (one block):
@@ -1331,10 +1330,9 @@ DevCSR transpose(const DevCSR& P, Pool& pool, Pool& scratch, cudaStream_t s) {
   R.m = P.n;
   R.nnz = P.nnz;
   int* cnt = scratch.alloc<int>(R.n + 1);
-  int* cursor = scratch.alloc<int>(R.n + 1);
+  int* place = scratch.alloc<int>(R.nnz + 1);
   TP_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int) * (R.n + 1), s));
-  TP_CUDA_TRY(cudaMemsetAsync(cursor, 0, sizeof(int) * (R.n + 1), s));
-  k_count_cols<<<grid_for(P.n), kBlock, 0, s>>>(P.n, P.rowptr, P.col, cnt);
+  k_count_cols<<<grid_for(P.n), kBlock, 0, s>>>(P.n, P.rowptr, P.col, cnt, place);
   TP_LAUNCH_CHECK();
   R.rowptr = pool.alloc<int>(R.n + 1);
   scan_exclusive(cnt, R.rowptr, R.n, scratch, s);
@@ -1344,7 +1342,7 @@ DevCSR transpose(const DevCSR& P, Pool& pool, Pool& scratch, cudaStream_t s) {
   int* ucol = scratch.alloc<int>(R.nnz + 1);
   double* uval = scratch.alloc<double>(R.nnz + 1);
   k_fill_transpose<<<grid_for(P.n), kBlock, 0, s>>>(P.n, P.rowptr, P.col, P.val, R.rowptr,
-                                                    cursor, ucol, uval);
+                                                    place, ucol, uval);
   TP_LAUNCH_CHECK();
   k_rank_rows<<<grid_for(R.n), kBlock, 0, s>>>(R.n, R.rowptr, ucol, uval, R.col, R.val);
   TP_LAUNCH_CHECK();
@@ -1365,7 +1363,9 @@ void csr_transpose_positions(const DevCSR& A, int* tpos, int* err, cudaStream_t 
   TP_LAUNCH_CHECK();
 }
 
-Hierarchy::~Hierarchy() = default;
+Hierarchy::~Hierarchy() {
+  for (cudaEvent_t e : phase_ev) cudaEventDestroy(e);
+}
 
 double Hierarchy::operator_complexity() const {
   if (L.empty() || L[0].A.nnz == 0) return 0.0;
@@ -1374,23 +1374,31 @@ double Hierarchy::operator_complexity() const {
   return s / L[0].A.nnz;
 }
 
-namespace {
-struct PhaseClock {
-  std::chrono::steady_clock::time_point t = std::chrono::steady_clock::now();
-  double lap(cudaStream_t s) {
-    TP_CUDA_TRY(cudaStreamSynchronize(s));
-    auto n = std::chrono::steady_clock::now();
-    double ms = std::chrono::duration<double, std::milli>(n - t).count();
-    t = n;
-    return ms;
+// phase boundaries as events on the setup's stream, read once at its end (a
+// host clock would need the stream to drain at each of them)
+void Hierarchy::mark_phase(int phase, cudaStream_t s) {
+  if (marks.size() == phase_ev.size()) {
+    cudaEvent_t e = nullptr;
+    TP_CUDA_TRY(cudaEventCreate(&e));
+    phase_ev.push_back(e);
   }
-};
-}  // namespace
+  TP_CUDA_TRY(cudaEventRecord(phase_ev[marks.size()], s));
+  marks.push_back(phase);
+}
+
+void Hierarchy::read_phases() {
+  for (double& x : phase_ms) x = 0.0;
+  for (size_t q = 1; q < marks.size(); ++q) {
+    float ms = 0.f;
+    TP_CUDA_TRY(cudaEventElapsedTime(&ms, phase_ev[q - 1], phase_ev[q]));
+    phase_ms[marks[q]] += ms;
+  }
+}
 
 void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
   opts = o;
-  for (double& x : phase_ms) x = 0.0;
-  PhaseClock clk;
+  marks.clear();
+  mark_phase(0, s);
   pool.release();
   scratch.release();
   L.clear();
@@ -1445,7 +1453,7 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
                                                  cur.cf);
     TP_LAUNCH_CHECK();
     // rounds are enqueued in batches (four, then pairs) before the host
-    // reads the count of undecided points: a round after the last is a no-op
+    // reads whether points are undecided: a round after the last is a no-op
     // (no point is undecided, so nothing is selected or changed); levels
     // here take about five rounds
     int rounds = 0;
@@ -1456,12 +1464,11 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
         ++rounds;
         if (wrow)
           k_pmis_select_warp<<<gw, kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.tpos, lam,
-                                                   cur.cf, opts.seed, newc);
+                                                   cur.cf, opts.seed, newc, undecided);
         else
           k_pmis_select<<<grid_for(n), kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.tpos,
-                                                       lam, cur.cf, opts.seed, newc);
+                                                       lam, cur.cf, opts.seed, newc, undecided);
         TP_LAUNCH_CHECK();
-        TP_CUDA_TRY(cudaMemsetAsync(undecided, 0, sizeof(int), s));
         if (wrow)
           k_pmis_update_warp<<<gw, kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.cf, newc,
                                                    undecided);
@@ -1473,12 +1480,9 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
       if (read_int(undecided, s) == 0) break;
     }
     cur.pmis_rounds = rounds;
-    phase_ms[0] += clk.lap(s);
-    int* flag = scratch.alloc<int>(n + 1);
+    mark_phase(0, s);
     int* cidx = scratch.alloc<int>(n + 1);
-    k_cflag<<<grid_for(n), kBlock, 0, s>>>(n, cur.cf, flag);
-    TP_LAUNCH_CHECK();
-    const int nc = (int)scan_exclusive(flag, cidx, n, scratch, s);
+    const int nc = (int)scan_states(cur.cf, kC, cidx, n, scratch, s);
     if (nc == 0 || (double)nc > 0.9 * (double)n) {
       cur.cf = nullptr;  // this level becomes the coarsest
       break;
@@ -1563,20 +1567,21 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
       P = T;
     }
     cur.P = P;
-    phase_ms[1] += clk.lap(s);
+    mark_phase(1, s);
     cur.R = transpose(P, pool, scratch, s);
-    phase_ms[2] += clk.lap(s);
+    mark_phase(2, s);
     cur.AP = csr_product(A, P, pool, scratch, s);
     DevCSR Ac = csr_product(cur.R, cur.AP, pool, scratch, s);
-    TP_CUDA_TRY(cudaStreamSynchronize(s));
-    phase_ms[3] += clk.lap(s);
+    mark_phase(3, s);
     scratch.release();
     L.emplace_back();
     L.back().A = Ac;
   }
-  clk.lap(s);
+  mark_phase(0, s);
   finish_levels(s, true);
-  phase_ms[4] += clk.lap(s);
+  mark_phase(4, s);
+  TP_CUDA_TRY(cudaStreamSynchronize(s));
+  read_phases();
 }
 
 // smoother scaling, FP32 copies, work vectors (allocate = first setup) and
@@ -1639,7 +1644,8 @@ void Hierarchy::finish_levels(cudaStream_t s, bool allocate) {
       v.ell_col = nullptr;
       v.ell_val = pool.alloc<double>((size_t)7 * n);
       v.ell_valf = f32 ? pool.alloc<float>((size_t)7 * n) : nullptr;
-    } else if (allocate && n >= 4096) {
+    } else if (allocate && n >= 4096 && v.A.nnz <= (long long)kEllMaxW * n) {
+      // (a longer mean row rules the copy out without the read-back)
       TP_CUDA_TRY(cudaMemsetAsync(err + 1, 0, sizeof(int), s));
       k_max_row<<<grid_for(n), kBlock, 0, s>>>(n, v.A.rowptr, err + 1);
       TP_LAUNCH_CHECK();
@@ -1729,7 +1735,8 @@ void Hierarchy::finish_levels(cudaStream_t s, bool allocate) {
     coarse_dense = pool.alloc<double>((size_t)nc * nc);
     coarse_inv = pool.alloc<double>((size_t)nc * nc);
   }
-  k_to_dense<<<grid_for(nc), kBlock, 0, s>>>(nc, cl.A.rowptr, cl.A.col, cl.A.val, coarse_dense);
+  TP_CUDA_TRY(cudaMemsetAsync(coarse_dense, 0, sizeof(double) * (size_t)nc * nc, s));
+  k_to_dense<<<grid_for((long long)nc * 32), kBlock, 0, s>>>(nc, cl.A.rowptr, cl.A.col, cl.A.val, coarse_dense);
   TP_LAUNCH_CHECK();
   TP_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), s));
   // one cluster holds the matrix in shared memory; the single-CTA kernel

@@ -147,9 +147,13 @@ void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s,
 
 // exclusive scan of n ints: out[0] = 0, out[i] = sum in[0..i-1]; out has
 // n + 1 entries and out[n] is the total. `in` and `out` may alias only if
-// equal. Returns the total (synchronises the stream).
-long long scan_exclusive(const int* in, int* out, int n, Pool& scratch,
-                         cudaStream_t s);
+// equal. Returns the total (synchronises the stream); with `extra`, a device
+// int as it stands then comes back in *extra_host.
+long long scan_exclusive(const int* in, int* out, int n, Pool& scratch, cudaStream_t s,
+                         const int* extra = nullptr, int* extra_host = nullptr);
+// the same over 1 where state[i] == what, else 0
+long long scan_states(const signed char* state, signed char what, int* out, int n, Pool& scratch,
+                      cudaStream_t s);
 
 // Deterministic sum of n doubles (fixed block partition and tree order),
 // result in *out (device).
