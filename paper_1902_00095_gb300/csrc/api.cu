@@ -1190,6 +1190,48 @@ void schur_diag_values(tp_ctx* c, bool symbolic) {
   TP_LAUNCH_CHECK();
 }
 
+// Work on the two hierarchies, which are independent: S~'s by a second host
+// thread on a second stream while this thread does A_pp's (setups and
+// refreshes are chains of small kernels with host round trips, so they
+// overlap; the four refreshes of a 64x64x32 Newton step one after the other
+// cost it 57 instead of 54 ms). Both see everything enqueued on the context stream before
+// the call, and it waits for both.
+template <class FP, class FS>
+static void on_both(tp_ctx* c, FP on_pp, FS on_S) {
+  cudaStream_t s = c->s;
+  if (!c->s2) {
+    TP_CUDA_TRY(cudaStreamCreateWithFlags(&c->s2, cudaStreamNonBlocking));
+    TP_CUDA_TRY(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
+    TP_CUDA_TRY(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
+  }
+  TP_CUDA_TRY(cudaEventRecord(c->ev_fork, s));
+  TP_CUDA_TRY(cudaStreamWaitEvent(c->s2, c->ev_fork, 0));
+  Error terr{TP_OK, ""};
+  bool tfail = false;
+  std::thread th([&]() {
+    try {
+      TP_CUDA_TRY(cudaSetDevice(c->device));
+      on_S(c->s2);
+    } catch (const Error& e) {
+      terr = e;
+      tfail = true;
+    } catch (...) {
+      terr = Error{TP_ECUDA, "Schur hierarchy setup failed"};
+      tfail = true;
+    }
+  });
+  try {
+    on_pp(s);
+  } catch (...) {
+    th.join();
+    throw;
+  }
+  th.join();
+  if (tfail) throw terr;
+  TP_CUDA_TRY(cudaEventRecord(c->ev_join, c->s2));
+  TP_CUDA_TRY(cudaStreamWaitEvent(s, c->ev_join, 0));
+}
+
 void build_device(tp_ctx* c, const tp_precond_opts& o) {
   cudaStream_t s = c->s;
   if (c->pc_graph) {
@@ -1245,40 +1287,8 @@ void build_device(tp_ctx* c, const tp_precond_opts& o) {
   } else if (o.smoother_S >= 0) {
     aS.smoother = o.smoother_S;
   }
-  // The two hierarchies are independent: S~'s is set up by a second host
-  // thread on a second stream while this thread sets up A_pp's (both setups
-  // are chains of small kernels with host round trips, so they overlap).
-  if (!c->s2) {
-    TP_CUDA_TRY(cudaStreamCreateWithFlags(&c->s2, cudaStreamNonBlocking));
-    TP_CUDA_TRY(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
-    TP_CUDA_TRY(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
-  }
-  TP_CUDA_TRY(cudaEventRecord(c->ev_fork, s));
-  TP_CUDA_TRY(cudaStreamWaitEvent(c->s2, c->ev_fork, 0));
-  Error terr{TP_OK, ""};
-  bool tfail = false;
-  std::thread th([&]() {
-    try {
-      TP_CUDA_TRY(cudaSetDevice(c->device));
-      c->hS->setup(S, aS, c->s2);
-    } catch (const Error& e) {
-      terr = e;
-      tfail = true;
-    } catch (...) {
-      terr = Error{TP_ECUDA, "Schur hierarchy setup failed"};
-      tfail = true;
-    }
-  });
-  try {
-    c->hpp->setup(App, ao, s);
-  } catch (...) {
-    th.join();
-    throw;
-  }
-  th.join();
-  if (tfail) throw terr;
-  TP_CUDA_TRY(cudaEventRecord(c->ev_join, c->s2));
-  TP_CUDA_TRY(cudaStreamWaitEvent(s, c->ev_join, 0));
+  on_both(c, [&](cudaStream_t t) { c->hpp->setup(App, ao, t); },
+          [&](cudaStream_t t) { c->hS->setup(S, aS, t); });
   c->hpp->probe = (c->probe_which == 0 || c->probe_which == 3) ? &c->probe : nullptr;
   c->hpp->probe_level = c->probe_which == 3 ? 1 : 0;
   c->hS->probe = c->probe_which == 1 ? &c->probe : nullptr;
@@ -1338,8 +1348,8 @@ void refresh_device(tp_ctx* c) {
                                   cudaMemcpyDeviceToDevice, s));
   }
   if (c->opts.schur == 3) schur_diag_values(c, false);
-  c->hpp->refresh(s);
-  c->hS->refresh(s);
+  on_both(c, [&](cudaStream_t t) { c->hpp->refresh(t); },
+          [&](cudaStream_t t) { c->hS->refresh(t); });
 }
 
 void negated_residual(tp_ctx* c) {
