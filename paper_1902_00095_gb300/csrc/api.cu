@@ -558,6 +558,18 @@ int tp_spmv(tp_ctx* c, const double* x_p, const double* x_T, double* y_p, double
   TP_API_BEGIN
   cudaStream_t s = c->s;
   const size_t n = c->N;
+  // device vectors are read and written in place unless an output overlaps an
+  // input (the four copies took a third of the call at 442 k cells)
+  const double* in[2] = {x_p, x_T};
+  double* out[2] = {y_p, y_T};
+  bool overlap = false;
+  for (const double* a : in)
+    for (const double* b : out) overlap = overlap || (a < b + n && b < a + n);
+  if (ptr_is_device && !overlap) {
+    tp::launch_block_spmv(c->N, c->rowptr, c->col, c->bval, x_p, x_T, y_p, y_T, nullptr, s);
+    TP_CUDA_TRY(cudaStreamSynchronize(s));
+    return TP_OK;
+  }
   to_device(c->io0, x_p, n, ptr_is_device, s);
   to_device(c->io1, x_T, n, ptr_is_device, s);
   tp::launch_block_spmv(c->N, c->rowptr, c->col, c->bval, c->io0, c->io1, c->io2, c->io3, nullptr,
