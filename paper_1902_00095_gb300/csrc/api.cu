@@ -129,6 +129,7 @@ void check_opts(const tp_precond_opts& o) {
 tp_ctx::~tp_ctx() {
   if (pc_graph) cudaGraphExecDestroy(pc_graph);
   if (pc_graph_tmpl) cudaGraphDestroy(pc_graph_tmpl);
+  if (vc_graph) cudaGraphExecDestroy(vc_graph);
   probe.destroy();
   hpp.reset();
   hS.reset();
@@ -1253,6 +1254,10 @@ void build_device(tp_ctx* c, const tp_precond_opts& o) {
   if (c->pc_graph_tmpl) {
     cudaGraphDestroy(c->pc_graph_tmpl);
     c->pc_graph_tmpl = nullptr;
+  }
+  if (c->vc_graph) {
+    cudaGraphExecDestroy(c->vc_graph);
+    c->vc_graph = nullptr;
   }
   c->probe_nodes.clear();
   c->probe_set = 0;

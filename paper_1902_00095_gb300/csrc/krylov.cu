@@ -29,6 +29,13 @@ namespace {
 constexpr int kDotWide = 8, kDotNarrow = 4;
 constexpr int kDotWideU = 2, kDotNarrowU = 4;  // elements a thread loads at a time
 constexpr long long kDotWideMaxN = 1ll << 20;  // vector length up to which 8 are taken
+// An iteration is enqueued before the host has seen the previous one's residual
+// estimate only while the last estimate it has seen is more than this factor
+// above the tolerance. Iterations reduce it 3- to 15-fold, so the last one is
+// not run ahead of and thrown away (an eighteenth iteration of 6.5 ms on the
+// layered 256x256x64 system, a fourteenth of 0.8 ms at 64x64x32), for a wait of
+// some 10 us at each of the last few.
+constexpr double kRunAhead = 20.0;
 constexpr int kEstSlot = 16;  // pinned-buffer offset of the two convergence-estimate slots
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -572,12 +579,15 @@ void ensure_workspace(tp_ctx* c, int restart) {
   c->restart_alloc = restart;
 }
 
-// y = A x (scalar CSR, one thread per row)
+// y = A x (scalar CSR, one thread per row); z = x
 __global__ void k_csr_spmv(int n, const int* __restrict__ rp, const int* __restrict__ col,
                            const double* __restrict__ val, const double* __restrict__ x,
-                           double* __restrict__ y) {
+                           double* __restrict__ z, double* __restrict__ y) {
+  pdl_wait();
+  pdl_trigger();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
+  z[i] = x[i];
   double a = 0.0;
   for (int e = rp[i]; e < rp[i + 1]; ++e) a += val[e] * x[col[e]];
   y[i] = a;
@@ -649,10 +659,51 @@ __global__ void k_column_schur(const int* __restrict__ rp, const int* __restrict
 
 }  // namespace
 
+// x_out = V(x_in) of the A_pp hierarchy inside a scalar solve: its V-cycle
+// captured as a graph at the first use after a build (about thirty kernels a
+// cycle; launched one by one, with a read-back per iteration, eight columns at
+// 32x32x16 took 10.3 ms, with the graph and scalar_fgmres's run-ahead 9.1)
+// unless the build asked for no graphs or its sweeps are being timed.
+static void scalar_vcycle(tp_ctx* c, Hierarchy& h, cudaStream_t s) {
+  if (!c->opts.use_graphs || h.probe) {
+    h.vcycle(s);
+    return;
+  }
+  if (!c->vc_graph) {
+    cudaGraph_t graph = nullptr;
+    TP_CUDA_TRY(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+    g_capturing = true;
+    try {
+      h.vcycle(s);
+    } catch (...) {
+      g_capturing = false;
+      cudaStreamEndCapture(s, &graph);
+      if (graph) cudaGraphDestroy(graph);
+      throw;
+    }
+    g_capturing = false;
+    TP_CUDA_TRY(cudaStreamEndCapture(s, &graph));
+    size_t nodes = 0;
+    cudaError_t e = cudaGraphGetNodes(graph, nullptr, &nodes);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&c->vc_graph, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) {
+      c->vc_graph = nullptr;
+      TP_CUDA_TRY(e);
+    }
+    c->vc_graph_kernels = (long long)nodes;  // every node is a kernel
+  }
+  TP_CUDA_TRY(cudaGraphLaunch(c->vc_graph, s));
+  count_launch(c->vc_graph_kernels);
+}
+
 // FGMRES(restart) on a scalar CSR system A x = b, right-preconditioned by
 // one V-cycle of h, x0 = 0, stop at ||b - A x|| <= rtol ||b||. Uses the
 // context's Krylov workspace. Returns the iteration count (negative when
-// rtol was not reached within maxit).
+// rtol was not reached within maxit). As in fgmres_solve, iteration j + 1 is
+// enqueued before the host looks at iteration j's estimate while the end is
+// far (kRunAhead); one enqueued past the stopping point touches nothing that
+// the columns before it use.
 int scalar_fgmres(tp_ctx* c, Hierarchy& h, const DevCSR& A, const double* b, double* x,
                   double rtol, int maxit, int restart) {
   cudaStream_t s = c->s;
@@ -674,43 +725,52 @@ int scalar_fgmres(tp_ctx* c, Hierarchy& h, const DevCSR& A, const double* b, dou
   TP_CUDA_TRY(cudaMemcpyAsync(c->hn, c->hn + 2, sizeof(double), cudaMemcpyDeviceToDevice, s));
   k_sqrt_inplace<<<1, 32, 0, s>>>(c->hn);
   TP_LAUNCH_CHECK();
+  auto enqueue = [&](int j) {
+    double* vj = c->Vb + (long long)j * n;
+    double* zj = c->Zb + (long long)j * n;
+    TP_CUDA_TRY(cudaMemcpyAsync(h.in, vj, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+    scalar_vcycle(c, h, s);
+    launch_pdl(k_csr_spmv, grid_for(n), kBlock, s, n, A.rowptr, A.col, A.val, h.out, zj, c->w);
+    double* h1 = c->h2;
+    double* h2 = c->h2 + (restart + 2);
+    const int G = orth_grid(c, n);
+    mdot_all(n, c->Vb, n, j + 1, c->w, c->kparts, B, h1, s);
+    launch_pdl(k_orth_update, G, 256, s, n, c->Vb, n, j + 1, h1, c->w, (double*)nullptr,
+               (const int*)nullptr);
+    mdot_all(n, c->Vb, n, j + 1, c->w, c->kparts, B, h2, s);
+    launch_pdl(k_orth_update, G, 256, s, n, c->Vb, n, j + 1, h2, c->w, c->oparts,
+               (const int*)nullptr);
+    launch_pdl(k_arnoldi, 1, 256, s, j, ldh, c->H, c->cs, c->sn, c->g, h1, h2, c->oparts, G,
+               c->hn, c->est);
+    TP_CUDA_TRY(cudaMemcpyAsync(hp_host + kEstSlot + 4 * (j & 1), c->est, 3 * sizeof(double),
+                                cudaMemcpyDeviceToHost, s));
+    TP_CUDA_TRY(cudaEventRecord(c->ev_est[j & 1], s));
+    if (j + 1 < restart)
+      launch_pdl(k_normalize, grid_for(n), kBlock, s, n, c->w, c->hn,
+                 c->Vb + (long long)(j + 1) * n);
+  };
   while (true) {
     if (beta <= rtol * bnorm) return its;
     if (its >= maxit) return -its;
     k_start_cycle<<<grid_for(n), kBlock, 0, s>>>(n, r, c->hn, c->Vb, c->g, restart);
     TP_LAUNCH_CHECK();
-    int m = 0;
+    int m = 0, queued = 0;
+    double seen = beta;
     for (int j = 0; j < restart; ++j) {
-      double* vj = c->Vb + (long long)j * n;
-      double* zj = c->Zb + (long long)j * n;
-      TP_CUDA_TRY(cudaMemcpyAsync(h.in, vj, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-      h.vcycle(s);
-      TP_CUDA_TRY(cudaMemcpyAsync(zj, h.out, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-      k_csr_spmv<<<grid_for(n), kBlock, 0, s>>>(n, A.rowptr, A.col, A.val, zj, c->w);
-      TP_LAUNCH_CHECK();
-      double* h1 = c->h2;
-      double* h2 = c->h2 + (restart + 2);
-      const int G = orth_grid(c, n);
-      mdot_all(n, c->Vb, n, j + 1, c->w, c->kparts, B, h1, s);
-      k_orth_update<<<G, 256, 0, s>>>(n, c->Vb, n, j + 1, h1, c->w, nullptr, nullptr);
-      TP_LAUNCH_CHECK();
-      mdot_all(n, c->Vb, n, j + 1, c->w, c->kparts, B, h2, s);
-      k_orth_update<<<G, 256, 0, s>>>(n, c->Vb, n, j + 1, h2, c->w, c->oparts, nullptr);
-      TP_LAUNCH_CHECK();
-      k_arnoldi<<<1, 256, 0, s>>>(j, ldh, c->H, c->cs, c->sn, c->g, h1, h2, c->oparts, G, c->hn,
-                                  c->est);
-      TP_LAUNCH_CHECK();
-      TP_CUDA_TRY(cudaMemcpyAsync(hp_host, c->est, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
-      TP_CUDA_TRY(cudaStreamSynchronize(s));
+      if (queued == j) enqueue(queued++);
+      if (j + 1 < restart && its + 1 < maxit && seen > kRunAhead * rtol * bnorm)
+        enqueue(queued++);
+      TP_CUDA_TRY(cudaEventSynchronize(c->ev_est[j & 1]));
+      const double* e = hp_host + kEstSlot + 4 * (j & 1);
+      const double est = e[0], hnv = e[1], den = e[2];
       ++its;
       m = j + 1;
-      if (!std::isfinite(hp_host[0]) || !(hp_host[2] > 0.0)) {
+      seen = est;
+      if (!std::isfinite(est) || !(den > 0.0)) {
         m = j;
         break;
       }
-      if (hp_host[0] <= rtol * bnorm || its >= maxit || hp_host[1] == 0.0) break;
-      k_normalize<<<grid_for(n), kBlock, 0, s>>>(n, c->w, c->hn, c->Vb + (long long)(j + 1) * n);
-      TP_LAUNCH_CHECK();
+      if (est <= rtol * bnorm || its >= maxit || hnv == 0.0) break;
     }
     if (m > 0) {
       k_hsolve<<<1, 32, 0, s>>>(m, ldh, c->H, c->g, c->yv);
@@ -861,12 +921,13 @@ int fgmres_solve(tp_ctx* c, const double* bp, const double* bT, double* xp, doub
       if (its >= maxit || breakdown) break;
       k_start_cycle<<<grid_for(n2), kBlock, 0, s>>>(n2, r, c->hn, c->Vb, c->g, restart);
       TP_LAUNCH_CHECK();
-      // Iteration j is enqueued before the host looks at iteration j - 1's
-      // convergence estimate (copied to pinned memory behind an event), so
-      // the GPU never idles on the host; an iteration enqueued past the
-      // stopping point is discarded (m counts checked columns only, and it
-      // touches nothing that columns < m use).
-      int m = 0;
+      // While the end is far (kRunAhead), iteration j is enqueued before the
+      // host looks at iteration j - 1's convergence estimate (copied to pinned
+      // memory behind an event), so the GPU does not idle on the host; an
+      // iteration enqueued past the stopping point is discarded (m counts
+      // checked columns only, and it touches nothing that columns < m use).
+      int m = 0, queued = 0;
+      double seen = beta;
       auto enqueue = [&](int j) {
         double* vj = c->Vb + (long long)j * n2;
         double* zj = c->Zb + (long long)j * n2;
@@ -914,6 +975,7 @@ int fgmres_solve(tp_ctx* c, const double* bp, const double* bT, double* xp, doub
         const double est = e[0], hnv = e[1], den = e[2];
         ++its;
         m = j + 1;
+        seen = est;
         if (!std::isfinite(est) || !std::isfinite(hnv) || !(den > 0.0)) {
           breakdown = true;  // drop the singular or non-finite column j
           m = j;
@@ -924,8 +986,9 @@ int fgmres_solve(tp_ctx* c, const double* bp, const double* bT, double* xp, doub
         return false;
       };
       for (int j = 0; j < restart; ++j) {
-        if (j == 0) enqueue(0);
-        if (j + 1 < restart && its + 1 < maxit) enqueue(j + 1);
+        if (queued == j) enqueue(queued++);
+        if (j + 1 < restart && its + 1 < maxit && seen > kRunAhead * rtol * bnorm)
+          enqueue(queued++);
         if (check(j)) break;
       }
       if (m > 0) {

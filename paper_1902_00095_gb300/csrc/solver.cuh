@@ -62,6 +62,10 @@ struct tp_ctx {
   std::vector<std::pair<cudaGraphNode_t, int>> probe_nodes;
   int probe_set = 0;
   long long pc_graph_kernels = 0;
+  // one V-cycle of the A_pp hierarchy (scalar solves of tp_probe_schur_columns),
+  // captured at the first such solve after a build
+  cudaGraphExec_t vc_graph = nullptr;
+  long long vc_graph_kernels = 0;
   // timing probe: -1 off, 0 finest A_pp sweeps, 1 finest S~ sweeps, 2 block SpMV
   int probe_which = -1;
   tp::Probe probe;
