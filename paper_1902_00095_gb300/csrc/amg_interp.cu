@@ -49,6 +49,9 @@ struct InterpWork {
 // class's capacities go to the next class through a list. Levels of at most
 // kInterpFewRows rows that are not short start at the last class, a warp per
 // row: the others would leave most SMs without a warp.
+// The last class takes rows of up to 128 strong F neighbours (32 at a time): one
+// row past it sends its level to the untruncated kernels (at 32 neighbours the
+// channelised 128x128x64 system had one: 46.0 instead of 44.1 ms a step).
 constexpr double kInterpShortMean = 20.0;
 constexpr int kInterpFewRows = 16384;
 
@@ -129,7 +132,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp(
     int* __restrict__ olist, int* __restrict__ ocnt) {
   using S = InterpRows<R, SET, ENT, KM, RL>;
   constexpr int HS = S::HS, NG = 32 / G, LR = 32 / R;
-  static_assert(KM <= G && R % NG == 0 && SET < kSelf && ENT < 0xffff, "capacities");
+  static_assert(KM < 256 && R % NG == 0 && SET < kSelf && ENT < 0xffff, "capacities");
   extern __shared__ __align__(16) char smem[];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   S& s = reinterpret_cast<S*>(smem)[w];
@@ -200,26 +203,33 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp(
           nk = 0;
         }
         __syncwarp();
-        // neighbour k on lane k: its row, its diagonal's sign
-        int kk = -1, kb = 0, klen = 0;
+        // G neighbours at a time, one on each lane: its row, its diagonal's sign
+        const int nk_max = __reduce_max_sync(kAll, nk);
+        int kk = -1, kb = 0, klen = 0, excl = 0, rel = 0, total = 0, total_max = 0;
         unsigned kc = 0;
-        if (gl < nk) {
-          kk = col[r0 + s.ke[r][gl]];
-          kb = rp[kk];
-          klen = rp[kk + 1] - kb;
-          kc = sign_class(val[dpos[kk]]);
-        }
-        int incl = klen;
+        auto load = [&](int k0) {
+          kk = -1;
+          kb = klen = 0;
+          kc = 0;
+          if (k0 + gl < nk) {
+            kk = col[r0 + s.ke[r][k0 + gl]];
+            kb = rp[kk];
+            klen = rp[kk + 1] - kb;
+            kc = sign_class(val[dpos[kk]]);
+          }
+          int incl = klen;
 #pragma unroll
-        for (int o = 1; o < G; o <<= 1) {
-          const int y = __shfl_up_sync(kAll, incl, o, G);
-          if (gl >= o) incl += y;
-        }
-        const int excl = incl - klen;
-        const int total = __shfl_sync(kAll, incl, G - 1, G);
-        const int total_max = __reduce_max_sync(kAll, total);
+          for (int o = 1; o < G; o <<= 1) {
+            const int y = __shfl_up_sync(kAll, incl, o, G);
+            if (gl >= o) incl += y;
+          }
+          excl = incl - klen;
+          rel = kb - excl;
+          total = __shfl_sync(kAll, incl, G - 1, G);
+          total_max = __reduce_max_sync(kAll, total);
+        };
+        load(0);
         // position p of the concatenated rows: owning neighbour and entry
-        const int rel = kb - excl;
         auto locate = [&](int p, int& own) -> int {
           int lo = 0;
 #pragma unroll
@@ -229,15 +239,18 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp(
           return __shfl_sync(kAll, rel, lo, G) + p;
         };
         if (EXT) {
-          for (int p0 = 0; p0 < total_max; p0 += G) {
-            const int p = p0 + gl;
-            int own;
-            const int f = locate(p, own);
-            const int kown = __shfl_sync(kAll, kk, own, G);
-            if (p < total && strong[f]) {
-              const int m = col[f];
-              if (m != kown && state[m] == kC)
-                hash_add<HS, SET>(s.hkey[r], s.setc[r], &s.ns[r], m);
+          for (int k0 = 0; k0 < nk_max; k0 += G) {
+            if (k0 > 0) load(k0);
+            for (int p0 = 0; p0 < total_max; p0 += G) {
+              const int p = p0 + gl;
+              int own;
+              const int f = locate(p, own);
+              const int kown = __shfl_sync(kAll, kk, own, G);
+              if (p < total && strong[f]) {
+                const int m = col[f];
+                if (m != kown && state[m] == kC)
+                  hash_add<HS, SET>(s.hkey[r], s.setc[r], &s.ns[r], m);
+              }
             }
           }
         }
@@ -268,7 +281,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp(
             s.num[r][gl + u * G] = 0.0;
             s.hslot[r][hash_find<HS>(s.hkey[r], key[u])] = (unsigned char)rank[u];
           }
-        if (gl < nk) s.kself[r][gl] = 0xffff;
+        for (int k = gl; k < nk; k += G) s.kself[r][k] = 0xffff;
         __syncwarp();
         // numerators start at a_im; a weak neighbour in the set is not lumped
         for (int e = gl; e < len; e += G) {
@@ -279,57 +292,62 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp(
           }
         }
         // the entries of the neighbours' rows that count, in order
-        int ne = 0, mine = 0;
-        for (int p0 = 0; p0 < total_max; p0 += G) {
-          const int p = p0 + gl;
-          int own;
-          const int f = locate(p, own);
-          const unsigned char okc = (unsigned char)__shfl_sync(kAll, kc, own, G);
-          bool sel = false;
-          double v = 0.0;
-          unsigned char slot = kSelf;
-          if (p < total && !over) {
-            v = val[f];
-            if (opposite_class(v, okc)) {
-              const int m = col[f];
-              if (EXT && m == i) {
-                sel = true;
-              } else {
-                const int h = hash_find<HS>(s.hkey[r], m);
-                if (h >= 0) {
+        int ne = 0;
+        for (int k0 = 0; k0 < nk_max; k0 += G) {
+          if (nk_max > G) load(k0);
+          const int ne0 = ne;
+          int mine = 0;
+          for (int p0 = 0; p0 < total_max; p0 += G) {
+            const int p = p0 + gl;
+            int own;
+            const int f = locate(p, own);
+            const unsigned char okc = (unsigned char)__shfl_sync(kAll, kc, own, G);
+            bool sel = false;
+            double v = 0.0;
+            unsigned char slot = kSelf;
+            if (p < total && !over) {
+              v = val[f];
+              if (opposite_class(v, okc)) {
+                const int m = col[f];
+                if (EXT && m == i) {
                   sel = true;
-                  slot = s.hslot[r][h];
+                } else {
+                  const int h = hash_find<HS>(s.hkey[r], m);
+                  if (h >= 0) {
+                    sel = true;
+                    slot = s.hslot[r][h];
+                  }
                 }
               }
             }
-          }
-          const unsigned bal = __ballot_sync(kAll, sel) & gmask;
-          if (sel) {
-            const int at = ne + __popc(bal & below);
-            if (at < ENT) {
-              s.ev[r][at] = v;
-              s.eslot[r][at] = slot;
-              s.ek[r][at] = (unsigned char)own;
-              if (slot == kSelf) s.kself[r][own] = (unsigned short)at;
+            const unsigned bal = __ballot_sync(kAll, sel) & gmask;
+            if (sel) {
+              const int at = ne + __popc(bal & below);
+              if (at < ENT) {
+                s.ev[r][at] = v;
+                s.eslot[r][at] = slot;
+                s.ek[r][at] = (unsigned char)(k0 + own);
+                if (slot == kSelf) s.kself[r][k0 + own] = (unsigned short)at;
+              }
+            }
+            ne += __popc(bal);
+            // entries of this lane's neighbour among the group's positions
+            const int lo = max(excl - p0, 0), hi = min(excl + klen - p0, G);
+            if (hi > lo) {
+              const unsigned bits = (bal >> (grp * G)) >> lo;
+              mine += __popc(hi - lo == 32 ? bits : bits & ((1u << (hi - lo)) - 1u));
             }
           }
-          ne += __popc(bal);
-          // entries of this lane's neighbour among the group's positions
-          const int lo = max(excl - p0, 0), hi = min(excl + klen - p0, G);
-          if (hi > lo) {
-            const unsigned bits = (bal >> (grp * G)) >> lo;
-            mine += __popc(hi - lo == 32 ? bits : bits & ((1u << (hi - lo)) - 1u));
+          int kincl = mine;
+#pragma unroll
+          for (int o = 1; o < G; o <<= 1) {
+            const int y = __shfl_up_sync(kAll, kincl, o, G);
+            if (gl >= o) kincl += y;
           }
+          if (k0 + gl < nk) s.kst[r][k0 + gl] = (unsigned short)min(ne0 + kincl - mine, ENT);
         }
         if (ne > ENT) over = true;
-        int kincl = mine;
-#pragma unroll
-        for (int o = 1; o < G; o <<= 1) {
-          const int y = __shfl_up_sync(kAll, kincl, o, G);
-          if (gl >= o) kincl += y;
-        }
         if (act && !over) {
-          if (gl < nk) s.kst[r][gl] = (unsigned short)(kincl - mine);
           if (gl == 0) {
             s.kst[r][nk] = (unsigned short)ne;
             s.nk[r] = nk;
@@ -528,7 +546,7 @@ void interp_tiers(const DevCSR& A, int sms, const int* dpos, const unsigned char
     list = w.olist1;
     nlist = w.ocnt + 1;
   }
-  launch_tier<EXT, 32, 1, 128, 1024, 32, 1024, 2>(6, sms, n, list, nlist, A, dpos, strong, state,
+  launch_tier<EXT, 32, 1, 128, 1024, 128, 1024, 2>(6, sms, n, list, nlist, A, dpos, strong, state,
                                                   cidx, pmax, w.cnt, w.tcol, w.tval, w.olist0,
                                                   w.ocnt + 2, s);
 }
