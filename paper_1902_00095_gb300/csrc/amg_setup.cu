@@ -70,193 +70,165 @@ __global__ void k_transpose_pos_warp(int n, const int* __restrict__ rp,
 // mean row length from which row-wise setup kernels take one warp per row
 constexpr int kWarpRowMean = 16;
 
-// strong[e] = 1 iff col != i and -a_e >= theta * max_{k != i}(-a_ik) > 0
-__global__ void k_strength(int n, const int* __restrict__ rp, const int* __restrict__ col,
-                           const double* __restrict__ val, double theta,
-                           unsigned char* __restrict__ strong) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double mx = -INFINITY;
-  for (int e = rp[i]; e < rp[i + 1]; ++e)
-    if (col[e] != i && -val[e] > mx) mx = -val[e];
-  if (!(mx > 0.0)) {
-    for (int e = rp[i]; e < rp[i + 1]; ++e) strong[e] = 0;
-    return;
-  }
-  const double thr = __dmul_rn(theta, mx);
-  for (int e = rp[i]; e < rp[i + 1]; ++e) strong[e] = (col[e] != i && -val[e] >= thr) ? 1 : 0;
-}
-
-__global__ void k_pmis_init(int n, const int* __restrict__ rp, const int* __restrict__ col,
-                            const unsigned char* __restrict__ strong,
-                            const int* __restrict__ tpos, int* __restrict__ lam,
-                            signed char* __restrict__ state) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int l = 0;
-  for (int e = rp[i]; e < rp[i + 1]; ++e)
-    if (col[e] != i && strong[tpos[e]]) ++l;
-  lam[i] = l;
-  state[i] = (l == 0) ? kF : kU;
-}
-
-__global__ void k_pmis_select(int n, const int* __restrict__ rp, const int* __restrict__ col,
-                              const unsigned char* __restrict__ strong,
-                              const int* __restrict__ tpos, const int* __restrict__ lam,
-                              const signed char* __restrict__ state, unsigned long long seed,
-                              unsigned char* __restrict__ newc, int* __restrict__ undecided) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) *undecided = 0;  // set again by this round's k_pmis_update
-  if (i >= n) return;
-  if (state[i] != kU) {
-    newc[i] = 0;
-    return;
-  }
-  const int li = lam[i];
-  const unsigned int hi = pmis_hash(seed, i);
-  unsigned char is_max = 1;
-  for (int e = rp[i]; e < rp[i + 1]; ++e) {
-    int k = col[e];
-    if (k == i || state[k] != kU) continue;
-    if (!(strong[e] || strong[tpos[e]])) continue;
-    int lk = lam[k];
-    unsigned int hk = pmis_hash(seed, k);
-    bool bigger = (lk > li) || (lk == li && (hk > hi || (hk == hi && k > i)));
-    if (bigger) {
-      is_max = 0;
-      break;
-    }
-  }
-  newc[i] = is_max;
-}
-
-__global__ void k_pmis_update(int n, const int* __restrict__ rp, const int* __restrict__ col,
-                              const unsigned char* __restrict__ strong,
-                              signed char* __restrict__ state,
-                              const unsigned char* __restrict__ newc,
-                              int* __restrict__ undecided) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  if (newc[i]) {
-    state[i] = kC;
-    return;
-  }
-  if (state[i] != kU) return;
-  for (int e = rp[i]; e < rp[i + 1]; ++e) {
-    int k = col[e];
-    if (strong[e] && (newc[k] || state[k] == kC)) {
-      state[i] = kF;
-      return;
-    }
-  }
-  *undecided = 1;  // the same value from every point that is left
-}
-
-// One-warp-per-row forms of the strength and PMIS kernels above, for levels
-// whose mean row length is at least kWarpRowMean: the lanes take the row's
-// entries, the row's decision is a warp reduction (a maximum, a count, an
-// any), so the results are the same bit for bit.
-__device__ __forceinline__ int warp_row(int& lane) {
-  lane = threadIdx.x & 31;
-  return (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
-}
-
-__global__ void k_strength_warp(int n, const int* __restrict__ rp, const int* __restrict__ col,
-                                const double* __restrict__ val, double theta,
-                                unsigned char* __restrict__ strong) {
-  int lane;
-  const int i = warp_row(lane);
-  if (i >= n) return;
-  const int r0 = rp[i], r1 = rp[i + 1];
-  double mx = -INFINITY;
-  for (int e = r0 + lane; e < r1; e += 32)
-    if (col[e] != i && -val[e] > mx) mx = -val[e];
+// Strength and PMIS take L lanes per row: 8 on short-row levels (the 7-point
+// finest, S~'s first Galerkin levels), a warp where the mean row length is at
+// least kWarpRowMean; a row's decision is a maximum, a count or an any over its
+// lanes.
+//
+// strong[e] = 1 iff col != i and -a_e >= theta * max_{k != i}(-a_ik) > 0. The
+// magnitudes of the negative entries are compared as integers (their bit
+// patterns order like the values): FP64 comparisons would take the FP64 pipe
+// for the whole warp (37 M entries of the layered A_pp's first Galerkin level
+// 868 us with them, a warp per row).
+template <int L>
+__global__ void __launch_bounds__(256) k_strength(int n, const int* __restrict__ rp,
+                                                  const int* __restrict__ col,
+                                                  const double* __restrict__ val, double theta,
+                                                  unsigned char* __restrict__ strong) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int i = (int)(t / L), lane = (int)(t % L);
+  const int r0 = i < n ? rp[i] : 0, r1 = i < n ? rp[i + 1] : 0;
+  // |a| of a negative entry off the diagonal (NaN and the others: 0)
+  auto key = [&](int e) -> unsigned long long {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(val[e]);
+    const unsigned long long m = u & 0x7fffffffffffffffull;
+    return (u >> 63) && m <= 0x7ff0000000000000ull && col[e] != i ? m : 0ull;
+  };
+  unsigned long long mx = 0;
+  for (int e = r0 + lane; e < r1; e += L) mx = max(mx, key(e));
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const double t = __shfl_xor_sync(0xffffffffu, mx, o);
-    if (t > mx) mx = t;
+  for (int o = L / 2; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  const unsigned long long thr = (unsigned long long)__double_as_longlong(
+      __dmul_rn(theta, __longlong_as_double((long long)mx)));
+  for (int e = r0 + lane; e < r1; e += L) {
+    bool s = false;
+    if (mx != 0) {
+      s = key(e) >= thr;
+      // a threshold that underflowed to zero is met by zeros, and by nothing
+      // positive, NaN or on the diagonal
+      if (thr == 0) {
+        const unsigned long long u = (unsigned long long)__double_as_longlong(val[e]);
+        s = col[e] != i && ((u << 1) == 0 || key(e) != 0);
+      }
+    }
+    strong[e] = s ? 1 : 0;
   }
-  if (!(mx > 0.0)) {
-    for (int e = r0 + lane; e < r1; e += 32) strong[e] = 0;
-    return;
-  }
-  const double thr = __dmul_rn(theta, mx);
-  for (int e = r0 + lane; e < r1; e += 32)
-    strong[e] = (col[e] != i && -val[e] >= thr) ? 1 : 0;
 }
 
-__global__ void k_pmis_init_warp(int n, const int* __restrict__ rp, const int* __restrict__ col,
-                                 const unsigned char* __restrict__ strong,
-                                 const int* __restrict__ tpos, int* __restrict__ lam,
-                                 signed char* __restrict__ state) {
-  int lane;
-  const int i = warp_row(lane);
-  if (i >= n) return;
+template <int L>
+__global__ void __launch_bounds__(256) k_pmis_init(int n, const int* __restrict__ rp,
+                                                   const int* __restrict__ col,
+                                                   const unsigned char* __restrict__ strong,
+                                                   const int* __restrict__ tpos,
+                                                   int* __restrict__ lam,
+                                                   signed char* __restrict__ state,
+                                                   unsigned char* __restrict__ newc) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int i = (int)(t / L), lane = (int)(t % L);
   int l = 0;
-  for (int e = rp[i] + lane; e < rp[i + 1]; e += 32)
-    if (col[e] != i && strong[tpos[e]]) ++l;
+  if (i < n)
+    for (int e = rp[i] + lane; e < rp[i + 1]; e += L)
+      if (col[e] != i && strong[tpos[e]]) ++l;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-  if (lane == 0) {
+  for (int o = L / 2; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+  if (i < n && lane == 0) {
     lam[i] = l;
     state[i] = (l == 0) ? kF : kU;
+    newc[i] = 0;
   }
 }
 
-__global__ void k_pmis_select_warp(int n, const int* __restrict__ rp,
-                                   const int* __restrict__ col,
-                                   const unsigned char* __restrict__ strong,
-                                   const int* __restrict__ tpos, const int* __restrict__ lam,
-                                   const signed char* __restrict__ state,
-                                   unsigned long long seed, unsigned char* __restrict__ newc,
-                                   int* __restrict__ undecided) {
-  int lane;
-  const int i = warp_row(lane);
-  if (i == 0 && lane == 0) *undecided = 0;  // set again by this round's update
-  if (i >= n) return;
-  if (state[i] != kU) {
-    if (lane == 0) newc[i] = 0;
-    return;
+// The undecided rows among the block's `rows` (at most 256), listed in shared
+// memory; returns their number. A round's kernels touch fewer and fewer rows:
+// with a lane group per row, decided or not, the rounds of the layered
+// 256x256x64 setups took 10.8 ms of kernel time, with the list 6.2.
+__device__ __forceinline__ int undecided_rows(int n, int rows,
+                                              const signed char* __restrict__ state, int* s_list,
+                                              int* s_warp) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * rows + threadIdx.x;
+  const bool und = (int)threadIdx.x < rows && i < n && state[i] == kU;
+  const unsigned m = __ballot_sync(0xffffffffu, und);
+  if (lane == 0) s_warp[warp] = __popc(m);
+  __syncthreads();
+  int before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    const int c = s_warp[w];
+    if (w < warp) before += c;
+    total += c;
   }
-  const int li = lam[i];
-  const unsigned int hi = pmis_hash(seed, i);
-  bool bigger = false;
-  for (int e = rp[i] + lane; e < rp[i + 1] && !bigger; e += 32) {
-    const int k = col[e];
-    if (k == i || state[k] != kU) continue;
-    if (!(strong[e] || strong[tpos[e]])) continue;
-    const int lk = lam[k];
-    const unsigned int hk = pmis_hash(seed, k);
-    bigger = (lk > li) || (lk == li && (hk > hi || (hk == hi && k > i)));
-  }
-  const bool any = __any_sync(0xffffffffu, bigger);
-  if (lane == 0) newc[i] = any ? 0 : 1;
+  if (und) s_list[before + __popc(m & ((1u << lane) - 1u))] = i;
+  __syncthreads();
+  return total;
 }
 
-__global__ void k_pmis_update_warp(int n, const int* __restrict__ rp,
-                                   const int* __restrict__ col,
-                                   const unsigned char* __restrict__ strong,
-                                   signed char* __restrict__ state,
-                                   const unsigned char* __restrict__ newc,
-                                   int* __restrict__ undecided) {
-  int lane;
-  const int i = warp_row(lane);
-  if (i >= n) return;
-  if (newc[i]) {
-    if (lane == 0) state[i] = kC;
-    return;
+// newc = 1 where an undecided point beats every undecided neighbour it is
+// strongly connected to, either way (decided points keep theirs: 1 for C, 0
+// for F)
+template <int L>
+__global__ void __launch_bounds__(256) k_pmis_select(
+    int n, const int* __restrict__ rp, const int* __restrict__ col,
+    const unsigned char* __restrict__ strong, const int* __restrict__ tpos,
+    const int* __restrict__ lam, const signed char* __restrict__ state, unsigned long long seed,
+    int rows, unsigned char* __restrict__ newc, int* __restrict__ undecided) {
+  __shared__ int s_list[256], s_warp[8];
+  if (blockIdx.x == 0 && threadIdx.x == 0) *undecided = 0;  // set again by k_pmis_update
+  const int m = undecided_rows(n, rows, state, s_list, s_warp);
+  constexpr int NG = 32 / L;  // rows a warp takes at a time
+  const int lane = threadIdx.x & 31, gl = lane % L;
+  for (int q0 = (threadIdx.x >> 5) * NG; q0 < m; q0 += 8 * NG) {
+    const int q = q0 + lane / L;
+    const int i = q < m ? s_list[q] : -1;
+    bool bigger = false;
+    if (i >= 0) {
+      const int li = lam[i];
+      const unsigned int hi = pmis_hash(seed, i);
+      for (int e = rp[i] + gl; e < rp[i + 1] && !bigger; e += L) {
+        const int k = col[e];
+        if (k == i || state[k] != kU) continue;
+        if (!(strong[e] || strong[tpos[e]])) continue;
+        const int lk = lam[k];
+        const unsigned int hk = pmis_hash(seed, k);
+        bigger = (lk > li) || (lk == li && (hk > hi || (hk == hi && k > i)));
+      }
+    }
+    const unsigned any = __ballot_sync(0xffffffffu, bigger) >> (lane - gl);
+    if (i >= 0 && gl == 0) newc[i] = (any & (L == 32 ? 0xffffffffu : (1u << L) - 1u)) ? 0 : 1;
   }
-  if (state[i] != kU) return;
-  bool c = false;
-  for (int e = rp[i] + lane; e < rp[i + 1] && !c; e += 32) {
-    const int k = col[e];
-    c = strong[e] && (newc[k] || state[k] == kC);
+}
+
+// new C points, and F where a point strongly depends on a C point; points left
+// undecided set *undecided, once per block
+template <int L>
+__global__ void __launch_bounds__(256) k_pmis_update(
+    int n, const int* __restrict__ rp, const int* __restrict__ col,
+    const unsigned char* __restrict__ strong, signed char* __restrict__ state, int rows,
+    const unsigned char* __restrict__ newc, int* __restrict__ undecided) {
+  __shared__ int s_list[256], s_warp[8];
+  const int m = undecided_rows(n, rows, state, s_list, s_warp);
+  constexpr int NG = 32 / L;
+  const int lane = threadIdx.x & 31, gl = lane % L;
+  bool left = false;
+  for (int q0 = (threadIdx.x >> 5) * NG; q0 < m; q0 += 8 * NG) {
+    const int q = q0 + lane / L;
+    const int i = q < m ? s_list[q] : -1;
+    const bool isc = i >= 0 && newc[i];
+    bool c = false;
+    if (i >= 0 && !isc)
+      for (int e = rp[i] + gl; e < rp[i + 1] && !c; e += L) {
+        const int k = col[e];
+        c = strong[e] && (newc[k] || state[k] == kC);
+      }
+    const unsigned any = (__ballot_sync(0xffffffffu, c) >> (lane - gl)) &
+                         (L == 32 ? 0xffffffffu : (1u << L) - 1u);
+    if (i >= 0 && gl == 0) {
+      if (isc) state[i] = kC;
+      else if (any) state[i] = kF;
+      else left = true;
+    }
   }
-  const bool any = __any_sync(0xffffffffu, c);
-  if (lane == 0) {
-    if (any) state[i] = kF;
-    else *undecided = 1;
-  }
+  if (__syncthreads_or(left) && threadIdx.x == 0) *undecided = 1;
 }
 
 // ---------------------------------------------------- classical interpolation
@@ -1434,11 +1406,11 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
     const bool wrow = A.nnz >= (long long)kWarpRowMean * n;
     const int gw = grid_for((long long)n * 32);
     cur.strong = pool.alloc<unsigned char>(A.nnz);
+    const int g8 = grid_for((long long)n * 8);
     if (wrow)
-      k_strength_warp<<<gw, kBlock, 0, s>>>(n, A.rowptr, A.col, A.val, opts.theta, cur.strong);
+      k_strength<32><<<gw, kBlock, 0, s>>>(n, A.rowptr, A.col, A.val, opts.theta, cur.strong);
     else
-      k_strength<<<grid_for(n), kBlock, 0, s>>>(n, A.rowptr, A.col, A.val, opts.theta,
-                                                cur.strong);
+      k_strength<8><<<g8, kBlock, 0, s>>>(n, A.rowptr, A.col, A.val, opts.theta, cur.strong);
     TP_LAUNCH_CHECK();
     // PMIS
     int* lam = scratch.alloc<int>(n);
@@ -1446,35 +1418,40 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
     int* undecided = scratch.alloc<int>(1);
     cur.cf = pool.alloc<signed char>(n);
     if (wrow)
-      k_pmis_init_warp<<<gw, kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.tpos, lam,
-                                             cur.cf);
+      k_pmis_init<32><<<gw, kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.tpos, lam, cur.cf,
+                                            newc);
     else
-      k_pmis_init<<<grid_for(n), kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.tpos, lam,
-                                                 cur.cf);
+      k_pmis_init<8><<<g8, kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.tpos, lam, cur.cf,
+                                           newc);
     TP_LAUNCH_CHECK();
     // rounds are enqueued in batches (four, then pairs) before the host
     // reads whether points are undecided: a round after the last is a no-op
     // (no point is undecided, so nothing is selected or changed); levels
     // here take about five rounds
+    // rows per block of 256 threads: all 256 where that leaves eight blocks per
+    // SM, fewer on small levels (at least one per lane group)
+    const int rows_min = wrow ? 8 : 32;
+    const int rows = std::max(rows_min, std::min(256, n / (8 * setup_sms())));
+    const int gr = grid_for(n, rows);
     int rounds = 0;
     while (true) {
       if (rounds >= opts.max_pmis_rounds) fail(TP_SETUP_FAILED, "PMIS round cap reached");
       const int batch = rounds == 0 ? 4 : 2;
       for (int r = 0; r < batch; ++r) {
         ++rounds;
-        if (wrow)
-          k_pmis_select_warp<<<gw, kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.tpos, lam,
-                                                   cur.cf, opts.seed, newc, undecided);
-        else
-          k_pmis_select<<<grid_for(n), kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.tpos,
-                                                       lam, cur.cf, opts.seed, newc, undecided);
-        TP_LAUNCH_CHECK();
-        if (wrow)
-          k_pmis_update_warp<<<gw, kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.cf, newc,
-                                                   undecided);
-        else
-          k_pmis_update<<<grid_for(n), kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.cf,
-                                                       newc, undecided);
+        if (wrow) {
+          k_pmis_select<32><<<gr, kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.tpos, lam,
+                                                  cur.cf, opts.seed, rows, newc, undecided);
+          TP_LAUNCH_CHECK();
+          k_pmis_update<32><<<gr, kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.cf, rows,
+                                                  newc, undecided);
+        } else {
+          k_pmis_select<8><<<gr, kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.tpos, lam,
+                                                 cur.cf, opts.seed, rows, newc, undecided);
+          TP_LAUNCH_CHECK();
+          k_pmis_update<8><<<gr, kBlock, 0, s>>>(n, A.rowptr, A.col, cur.strong, cur.cf, rows,
+                                                 newc, undecided);
+        }
         TP_LAUNCH_CHECK();
       }
       if (read_int(undecided, s) == 0) break;
