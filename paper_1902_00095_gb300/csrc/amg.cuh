@@ -181,6 +181,16 @@ class Hierarchy {
   void refresh(cudaStream_t s);
   // One V-cycle: out = V(in). in/out are the hierarchy's own FP64 buffers.
   void vcycle(cudaStream_t s);
+  // The same on another set of work vectors, so that cycles can run side by
+  // side on streams of their own: levels and buffers from second_set(), whose
+  // memory comes from `p`; valid until the next setup (a refresh keeps it).
+  // Not available with a cluster tail (empty levels).
+  struct WorkSet {
+    std::vector<Level> L;
+    double *in = nullptr, *out = nullptr;
+  };
+  WorkSet second_set(Pool& p) const;
+  void vcycle(WorkSet& w, cudaStream_t s);
   double operator_complexity() const;
   // algorithmic bytes of one V-cycle (each kernel's operator, scaling and
   // vectors counted once)
@@ -216,8 +226,7 @@ class Hierarchy {
   void read_phases();
   void finish_levels(cudaStream_t s, bool allocate);
   void plan_tail(cudaStream_t s);
-  void vcycle_fp64(cudaStream_t s);
-  void vcycle_fp32(cudaStream_t s);
+  void vcycle_on(std::vector<Level>& levels, const double* b, double* x, cudaStream_t s);
 };
 
 // Chebyshev smoother (chebyshev.cu): plain-diagonal scaling, lambda_max by

@@ -126,21 +126,6 @@ void check_opts(const tp_precond_opts& o) {
 
 }  // namespace
 
-tp_ctx::~tp_ctx() {
-  if (pc_graph) cudaGraphExecDestroy(pc_graph);
-  if (pc_graph_tmpl) cudaGraphDestroy(pc_graph_tmpl);
-  if (vc_graph) cudaGraphExecDestroy(vc_graph);
-  probe.destroy();
-  hpp.reset();
-  hS.reset();
-  if (host_est) cudaFreeHost(host_est);
-  if (ev_fork) cudaEventDestroy(ev_fork);
-  for (cudaEvent_t e : ev_est)
-    if (e) cudaEventDestroy(e);
-  if (ev_join) cudaEventDestroy(ev_join);
-  if (s2) cudaStreamDestroy(s2);
-}
-
 struct tp_amg {
   cudaStream_t s = nullptr;
   bool own_stream = false;
@@ -962,6 +947,13 @@ int tp_probe_schur_columns(tp_ctx* c, const int* cols, int ncols, double rtol, i
   if (!c || !cols || ncols < 0 || !entry || !value || !(rtol > 0.0)) return TP_EINVAL;
   if (!c->built) return TP_ESTATE;
   TP_API_BEGIN
+  if (tp::column_lanes_usable(c, ncols)) {
+    int good = 0;  // columns before the first index out of range
+    while (good < ncols && cols[good] >= 0 && cols[good] < c->N) ++good;
+    const int st = tp::probe_schur_columns_lanes(c, cols, good, rtol, 500, entry, value,
+                                                 good < ncols ? nullptr : iters);
+    return good < ncols ? TP_EINVAL : st;
+  }
   int* d_entry = reinterpret_cast<int*>(c->io2);
   double* d_val = c->io3;
   int total = 0, status = TP_OK;
@@ -1259,6 +1251,7 @@ void build_device(tp_ctx* c, const tp_precond_opts& o) {
     cudaGraphExecDestroy(c->vc_graph);
     c->vc_graph = nullptr;
   }
+  stale_column_lanes(c);
   c->probe_nodes.clear();
   c->probe_set = 0;
   c->built = false;

@@ -5,6 +5,10 @@
 #include "kernels.cuh"
 #include "learned.cuh"
 
+namespace tp {
+struct ColumnLane;  // krylov.cu
+}
+
 struct tp_ctx {
   cudaStream_t s = nullptr;
   int device = 0;
@@ -66,6 +70,9 @@ struct tp_ctx {
   // captured at the first such solve after a build
   cudaGraphExec_t vc_graph = nullptr;
   long long vc_graph_kernels = 0;
+  // workspaces of Schur columns solved side by side
+  std::vector<std::unique_ptr<tp::ColumnLane>> lanes;
+  cudaEvent_t ev_lanes = nullptr;
   // timing probe: -1 off, 0 finest A_pp sweeps, 1 finest S~ sweeps, 2 block SpMV
   int probe_which = -1;
   tp::Probe probe;
@@ -93,6 +100,7 @@ struct tp_ctx {
   // user-facing scratch for host pointer marshalling
   double *io0 = nullptr, *io1 = nullptr, *io2 = nullptr, *io3 = nullptr;
 
+  tp_ctx();
   ~tp_ctx();
 };
 
@@ -116,5 +124,11 @@ int newton_step(tp_ctx* c, double dt, const tp_precond_opts& popts, const tp_new
 int scalar_fgmres(tp_ctx* c, Hierarchy& h, const DevCSR& A, const double* b, double* x,
                   double rtol, int maxit, int restart);
 int probe_schur_column(tp_ctx* c, int j, double rtol, int maxit, int* entry, double* value);
+// the same for several columns side by side: host outputs, total iterations;
+// TP_OK or TP_NOT_CONVERGED
+bool column_lanes_usable(const tp_ctx* c, int ncols);
+int probe_schur_columns_lanes(tp_ctx* c, const int* cols, int ncols, double rtol, int maxit,
+                              int* entry, double* value, int* iters);
+void stale_column_lanes(tp_ctx* c);
 void learned_features(tp_ctx* c);  // features of the last assembly into c->feat
 }  // namespace tp

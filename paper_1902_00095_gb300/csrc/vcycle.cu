@@ -958,23 +958,35 @@ TV* run_level(std::vector<Level>& L, const double* cinv, size_t l, const TB* b, 
 
 }  // namespace
 
-void Hierarchy::vcycle(cudaStream_t s) {
-  if (opts.precision >= 1) vcycle_fp32(s);
-  else vcycle_fp64(s);
-}
+void Hierarchy::vcycle(cudaStream_t s) { vcycle_on(L, in, out, s); }
 
-void Hierarchy::vcycle_fp64(cudaStream_t s) {
+void Hierarchy::vcycle(WorkSet& w, cudaStream_t s) { vcycle_on(w.L, w.in, w.out, s); }
+
+void Hierarchy::vcycle_on(std::vector<Level>& levels, const double* b, double* x,
+                          cudaStream_t s) {
   Smooth sm{opts.smoother, opts.cheb_degree, tail_first, tail_cluster, nc, tail_desc,
             opts.line_nxy, opts.line_nz, opts.nu_line, probe_level};
-  run_level<double, double, double>(L, coarse_inv, 0, in, out, opts.nu_pre, opts.nu_post, sm, s,
-                                    probe);
+  if (opts.precision >= 1)
+    run_level<float, double, double>(levels, coarse_inv, 0, b, x, opts.nu_pre, opts.nu_post, sm,
+                                     s, probe);
+  else
+    run_level<double, double, double>(levels, coarse_inv, 0, b, x, opts.nu_pre, opts.nu_post, sm,
+                                      s, probe);
 }
 
-void Hierarchy::vcycle_fp32(cudaStream_t s) {
-  Smooth sm{opts.smoother, opts.cheb_degree, tail_first, tail_cluster, nc, tail_desc,
-            opts.line_nxy, opts.line_nz, opts.nu_line, probe_level};
-  run_level<float, double, double>(L, coarse_inv, 0, in, out, opts.nu_pre, opts.nu_post, sm, s,
-                                   probe);
+Hierarchy::WorkSet Hierarchy::second_set(Pool& p) const {
+  WorkSet w;
+  if (tail_first >= 0) return w;
+  w.L = L;
+  const size_t es = opts.precision >= 1 ? sizeof(float) : sizeof(double);
+  for (Level& v : w.L) {
+    for (void** q : {&v.b, &v.x, &v.t, &v.r}) *q = p.alloc<char>(es * (v.A.n + 1));
+    if (opts.smoother == 1)
+      for (void** q : {&v.cw, &v.cd0, &v.cd1, &v.cr}) *q = p.alloc<char>(es * (v.A.n + 1));
+  }
+  w.in = p.alloc<double>(n0 + 1);
+  w.out = p.alloc<double>(n0 + 1);
+  return w;
 }
 
 // ------------------------------------------------- V-cycle byte count
