@@ -142,7 +142,11 @@ __device__ __forceinline__ void mlp_forward_tile(const MlpDev& m, const float* _
 
 // Training: forward + backward of 16 samples per warp; writes the warp's
 // gradient partial (kMlpParams floats) and loss partial to partials[tile].
-constexpr int kTrainWarps = 4;
+// One warp per block: the kernel is bound by the latency of a warp's chain
+// through the layers, and 256 tiles then spread over all SMs (14.8 us; four
+// warps per block on 64 SMs 20.1, the weight gradients of a tile split over
+// four warps 17.8: 255 registers leave room for few warps).
+constexpr int kTrainWarps = 1;
 
 __global__ void __launch_bounds__(32 * kTrainWarps) k_mlp_train_tile(
     MlpDev m, int B, const float* __restrict__ X, const int* __restrict__ slot,
@@ -329,30 +333,69 @@ __global__ void __launch_bounds__(32 * kTrainWarps) k_mlp_train_tile(
 }
 
 // grad[p] = sum over tiles of partials[tile][p] (fixed order); the loss in
-// grad[kMlpParams]
-__global__ void k_mlp_reduce(int ntiles, const float* __restrict__ partials,
-                             float* __restrict__ grad) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p > kMlpParams) return;
-  float s = 0.f;
-  for (int k = 0; k < ntiles; ++k) s += partials[(size_t)k * kMlpPartial + p];
-  grad[p] = s;
-}
+// grad[kMlpParams]. ADAM: then one step (Kingma and Ba 2015, bias-corrected,
+// FP32 master weights) and the weight's BF16 copies, each parameter by the
+// thread that summed it (three kernels before). The sum is serial in the
+// tiles, so a block brings kRedTiles tiles of its 32 parameters into shared
+// memory at once and adds from there: 256 tiles 9.1 us with a thread's loads
+// four at a time.
+constexpr int kRedTiles = 256;
 
-// Adam (Kingma and Ba 2015), bias-corrected, FP32 master weights
-__global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ mm,
-                       float* __restrict__ vv, int step, float lr) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= kMlpParams) return;
+template <bool ADAM>
+__global__ void __launch_bounds__(256) k_mlp_reduce(int ntiles,
+                                                    const float* __restrict__ partials,
+                                                    float* __restrict__ grad, MlpDev m, int step,
+                                                    float lr) {
+  __shared__ float sh[kRedTiles][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int p = blockIdx.x * 32 + lane;
+  float s = 0.f;
+  for (int k0 = 0; k0 < ntiles; k0 += kRedTiles) {
+    const int nk = min(kRedTiles, ntiles - k0);
+    float v[kRedTiles / 8];
+#pragma unroll
+    for (int u = 0; u < kRedTiles / 8; ++u) {
+      const int k = u * 8 + warp;
+      v[u] = k < nk && p <= kMlpParams ? partials[(size_t)(k0 + k) * kMlpPartial + p] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < kRedTiles / 8; ++u) sh[u * 8 + warp][lane] = v[u];
+    __syncthreads();
+    if (warp == 0)
+      for (int k = 0; k < nk; ++k) s += sh[k][lane];
+    __syncthreads();
+  }
+  if (warp != 0 || p > kMlpParams) return;
+  grad[p] = s;
+  if (!ADAM || p >= kMlpParams) return;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  const float gi = g[p];
-  const float mi = b1 * mm[p] + (1.f - b1) * gi;
-  const float vi = b2 * vv[p] + (1.f - b2) * gi * gi;
-  mm[p] = mi;
-  vv[p] = vi;
+  const float gi = s;
+  const float mi = b1 * m.adam_m[p] + (1.f - b1) * gi;
+  const float vi = b2 * m.adam_v[p] + (1.f - b2) * gi * gi;
+  m.adam_m[p] = mi;
+  m.adam_v[p] = vi;
   const float mh = mi / (1.f - powf(b1, (float)step));
   const float vh = vi / (1.f - powf(b2, (float)step));
-  w[p] -= lr * mh / (sqrtf(vh) + eps);
+  float w = m.params[p];
+  w -= lr * mh / (sqrtf(vh) + eps);
+  m.params[p] = w;
+  // the places of weight p in the BF16 copies (k_mlp_pack; their padding stays)
+  const __nv_bfloat16 h = __float2bfloat16_rn(w);
+  if (p < kOffB1) {
+    const int o = p / kMlpIn, i = p % kMlpIn;
+    m.W1[o * kMlpInPad + i] = h;
+    m.Wtc[mlp_core_off(o, i, 32) / 2] = h;
+  } else if (p >= kOffW2 && p < kOffB2) {
+    const int q = p - kOffW2, o = q / kMlpHidden, i = q % kMlpHidden;
+    m.W2[q] = h;
+    m.W2T[i * kMlpHidden + o] = h;
+    m.Wtc[64 * 32 + mlp_core_off(o, i, 64) / 2] = h;
+  } else if (p >= kOffW3 && p < kOffB3) {
+    const int q = p - kOffW3, o = q / kMlpHidden, i = q % kMlpHidden;
+    m.W3[q] = h;
+    m.W3T[i * 16 + o] = h;
+    m.Wtc[64 * 32 + 64 * 64 + mlp_core_off(o, i, 64) / 2] = h;
+  }
 }
 
 // BF16 copies used by the tensor-core kernels
@@ -459,22 +502,33 @@ void mlp_forward(const MlpDev& m, int n, const float* X, float* O, cudaStream_t 
   if (h != 0) fail(TP_ECUDA, "MLP forward: a tensor-core completion wait timed out");
 }
 
-void mlp_gradient(const MlpDev& m, int B, const float* X, const int* slot, const double* St,
-                  const double* Sd, const double* target, float* partials, float* grad,
-                  cudaStream_t s) {
+// the tiles' gradients of a batch
+static int mlp_tiles(const MlpDev& m, int B, const float* X, const int* slot, const double* St,
+                     const double* Sd, const double* target, float* partials, cudaStream_t s) {
   const int tiles = (B + 15) / 16;
   k_mlp_train_tile<<<(tiles + kTrainWarps - 1) / kTrainWarps, 32 * kTrainWarps, 0, s>>>(
       m, B, X, slot, St, Sd, target, partials);
   TP_LAUNCH_CHECK();
-  k_mlp_reduce<<<grid_for(kMlpParams + 1), kBlock, 0, s>>>(tiles, partials, grad);
+  return tiles;
+}
+
+void mlp_gradient(const MlpDev& m, int B, const float* X, const int* slot, const double* St,
+                  const double* Sd, const double* target, float* partials, float* grad,
+                  cudaStream_t s) {
+  const int tiles = mlp_tiles(m, B, X, slot, St, Sd, target, partials, s);
+  k_mlp_reduce<false><<<grid_for(kMlpParams + 1, 32), 256, 0, s>>>(tiles, partials, grad, m, 0,
+                                                                   0.f);
   TP_LAUNCH_CHECK();
 }
 
-void mlp_adam(MlpDev& m, const float* grad, float lr, cudaStream_t s) {
+void mlp_train_step(MlpDev& m, int B, const float* X, const int* slot, const double* St,
+                    const double* Sd, const double* target, float* partials, float* grad,
+                    float lr, cudaStream_t s) {
+  const int tiles = mlp_tiles(m, B, X, slot, St, Sd, target, partials, s);
   m.step += 1;
-  k_adam<<<grid_for(kMlpParams), kBlock, 0, s>>>(m.params, grad, m.adam_m, m.adam_v, m.step, lr);
+  k_mlp_reduce<true><<<grid_for(kMlpParams + 1, 32), 256, 0, s>>>(tiles, partials, grad, m, m.step,
+                                                                  lr);
   TP_LAUNCH_CHECK();
-  mlp_pack(m, s);
 }
 
 }  // namespace tp

@@ -51,7 +51,10 @@ void mlp_forward_tc(const MlpDev& m, int n, const float* X, float* O, int* err, 
 void mlp_gradient(const MlpDev& m, int B, const float* X, const int* slot, const double* St,
                   const double* Sd, const double* target, float* partials, float* grad,
                   cudaStream_t s);
-void mlp_adam(MlpDev& m, const float* grad, float lr, cudaStream_t s);
+// the same gradient, then one Adam step of learning rate lr
+void mlp_train_step(MlpDev& m, int B, const float* X, const int* slot, const double* St,
+                    const double* Sd, const double* target, float* partials, float* grad,
+                    float lr, cudaStream_t s);
 
 // learned S~ values on the 7-point pattern with the per-row guard; returns
 // (through *nbad, device int) the number of rows that fell back
