@@ -34,7 +34,7 @@ namespace tp {
 
 namespace {
 
-constexpr int kGjThreads = 1024;
+constexpr int kGjThreads = 512;
 constexpr int kGjWarps = kGjThreads / 32;
 
 // shared-memory layout of one CTA (R rows of n entries), same on both sides
