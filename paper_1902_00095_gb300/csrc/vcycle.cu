@@ -452,6 +452,109 @@ __global__ void __launch_bounds__(128) k_line_sweep(
   }
 }
 
+// The same step by blocks of W columns: the residual rows of all layers are
+// formed by all threads at once (coalesced over the columns) into shared
+// memory together with the columns' factors, one warp then runs the two
+// recurrences of every column from there, and all threads write x_in + e. The
+// operations of a cell and their order are those of k_line_sweep, whose two
+// threads per column form each residual row inside the recurrence: a chain of
+// about 1 us per layer that leaves the GPU idle on small grids and never fills
+// it on large ones.
+constexpr int kLineThreads = 256;
+constexpr int kLineFewBlocks = 152;           // blocks of 16 columns that reach every SM
+constexpr int kLineManyColumns = 152 * 128;   // columns that k_line_sweep fills the GPU with
+constexpr size_t kLineSmemShare = 16 << 10;   // of a block, eight blocks per SM
+constexpr size_t kLineSmemMax = 200 << 10;    // of a block
+
+template <class TV>
+size_t line_block_smem(int nz, int W) {
+  return (size_t)4 * nz * W * sizeof(TV);
+}
+
+template <int W, class TV, class TB, class TO>
+__global__ void __launch_bounds__(kLineThreads) k_line_block(
+    int nxy, int nz, int n, int ell_w, const int* __restrict__ ecol, int snx, int snxy,
+    const TV* __restrict__ eval, const int* __restrict__ rp, const int* __restrict__ col,
+    const TV* __restrict__ val, const TV* __restrict__ lo, const TV* __restrict__ minv,
+    const TV* __restrict__ cp, const TB* __restrict__ b, const TV* __restrict__ xin,
+    TO* __restrict__ xout) {
+  static_assert(2 * W <= 32, "both ends of a block's columns in one warp");
+  extern __shared__ __align__(16) char s_line[];
+  TV* sr = reinterpret_cast<TV*>(s_line);  // [nz][W]: residuals, g, then e
+  TV* sl = sr + nz * W;
+  TV* sm = sl + nz * W;
+  TV* sc = sm + nz * W;
+  const int cl = threadIdx.x % W, c = blockIdx.x * W + cl;
+  const bool act = c < nxy;
+  pdl_wait();
+  pdl_trigger();
+  for (int z = threadIdx.x / W; z < nz; z += kLineThreads / W) {
+    if (!act) break;
+    const int i = c + z * nxy, q = z * W + cl;
+    TV r = (TV)b[i];
+    sl[q] = lo[i];
+    sm[q] = minv[i];
+    sc[q] = cp[i];
+    if (xin) {
+      TV ax = TV(0);
+      if (ell_w > 0) {
+#pragma unroll
+        for (int k = 0; k < kEllMaxW; ++k)
+          if (k < ell_w) {
+            const long long e = (long long)k * n + i;
+            ax += eval[e] * xin[ecol ? ecol[e] : stencil_col(k, i, n, snx, snxy)];
+          }
+      } else {
+        for (int e = rp[i]; e < rp[i + 1]; ++e) ax += val[e] * xin[col[e]];
+      }
+      r -= ax;
+    }
+    sr[q] = r;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    // lanes 0..W-1 the top rows, W..2W-1 the bottom rows
+    const int role = (threadIdx.x / W) & 1;
+    const bool on = act && threadIdx.x < 2 * W;
+    const int mid = nz >> 1;
+    const int nsteps = role ? nz - 1 - mid : mid;
+    TV gprev = TV(0);
+#pragma unroll 4
+    for (int s = 0; s < mid; ++s)
+      if (on && s < nsteps) {
+        const int q = (role ? nz - 1 - s : s) * W + cl;
+        const TV g = (sr[q] - sl[q] * gprev) * sm[q];
+        sr[q] = g;
+        gprev = g;
+      }
+    const TV gb = __shfl_down_sync(0xffffffffu, gprev, W);
+    TV xm = TV(0);
+    if (on && role == 0) {
+      const int q = mid * W + cl;
+      const TV gt = mid > 0 ? gprev : TV(0);
+      const TV gu = mid + 1 < nz ? gb : TV(0);
+      xm = (sr[q] - sl[q] * gt - sc[q] * gu) * sm[q];
+      sr[q] = xm;
+    }
+    TV enext = __shfl_sync(0xffffffffu, xm, cl);
+#pragma unroll 4
+    for (int s = 0; s < mid; ++s)
+      if (on && s < nsteps) {
+        const int q = (role ? mid + 1 + s : mid - 1 - s) * W + cl;
+        const TV e = sr[q] - sc[q] * enext;
+        sr[q] = e;
+        enext = e;
+      }
+  }
+  __syncthreads();
+  for (int z = threadIdx.x / W; z < nz; z += kLineThreads / W) {
+    if (!act) break;
+    const int i = c + z * nxy;
+    const TV e = sr[z * W + cl];
+    xout[i] = (TO)(xin ? xin[i] + e : e);
+  }
+}
+
 // Sliced-ELL forms (levels below the finest with long rows): one thread per
 // row in length-sorted order, one warp per 32-row slice, so a warp loads 32
 // consecutive entries at each step and its lanes idle only on the slice's
@@ -805,11 +908,42 @@ double line_bytes(const Level& v, bool from_zero) {
   return bytes;
 }
 
+template <int W, class TV, class TB, class TO>
+void line_block(const Smooth& sm, const Level& v, const TB* b, const TV* xin, TO* xout,
+                cudaStream_t s) {
+  auto kern = k_line_block<W, TV, TB, TO>;
+  static const bool attr = [&]() {
+    TP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kLineSmemMax));
+    return true;
+  }();
+  (void)attr;
+  launch_pdl_smem(kern, (sm.line_nxy + W - 1) / W, kLineThreads,
+                  line_block_smem<TV>(sm.line_nz, W), s, sm.line_nxy, sm.line_nz, v.A.n, v.ell_w,
+                  v.ell_col, v.ell_nx, v.ell_nxy, Vals<TV>::E(v), v.A.rowptr, v.A.col,
+                  Vals<TV>::A(v), Vals<TV>::lo(v), Vals<TV>::minv(v), Vals<TV>::cp(v), b, xin,
+                  xout);
+}
+
 template <class TV, class TB, class TO>
 void line_step(const Smooth& sm, const Level& v, const TB* b, const TV* xin, TO* xout,
                cudaStream_t s) {
-  // two threads per column; small blocks spread a few thousand columns over
-  // every SM
+  // Blocks of 16 columns while eight of them leave half of an SM's memory to the
+  // L1 cache, else of 8: a larger share of shared memory stays in force for the
+  // kernels that follow, whose gathers live in L1 (FP64 256x256x64 with blocks
+  // of 16, 32 KB each: this kernel 3.7 ms a solve and the other kernels 105.1,
+  // with blocks of 8, 16 KB each: 3.8 and 100.8). Columns too long for that go
+  // to k_line_sweep where it has enough of them, and to it in any case past
+  // kLineSmemMax.
+  const size_t s16 = line_block_smem<TV>(sm.line_nz, 16), s8 = s16 / 2;
+  if (s16 <= kLineSmemShare && sm.line_nxy >= 16 * kLineFewBlocks) {
+    line_block<16, TV, TB, TO>(sm, v, b, xin, xout, s);
+    return;
+  }
+  if (s8 <= kLineSmemShare || (s8 <= kLineSmemMax && sm.line_nxy < kLineManyColumns)) {
+    line_block<8, TV, TB, TO>(sm, v, b, xin, xout, s);
+    return;
+  }
   const long long lanes = 2ll * sm.line_nxy;
   const int threads = lanes >= 152 * 128 * 2 ? 128 : 32;
   const int grid = (int)((lanes + threads - 1) / threads);
