@@ -5,6 +5,7 @@
 #include <cstring>
 #include <algorithm>
 #include <thread>
+#include <cuda.h>
 #include "solver.cuh"
 
 using tp::Error;
@@ -174,6 +175,33 @@ struct tp_mlp {
 };
 
 namespace {
+// Whether a kernel may use the caller's array where it lies: device memory,
+// aligned to its type, `n` elements inside one allocation. A copy accepts any
+// address and reports what it cannot reach, so everything else goes through one.
+template <class T>
+bool usable_in_place(const T* p, size_t n) {
+  using Query = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Query query = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault,
+                                         &r) != cudaSuccess)
+      cudaGetLastError();
+    return reinterpret_cast<Query>(f);
+  }();
+  const auto at = reinterpret_cast<uintptr_t>(p);
+  if (!query || at % alignof(T)) return false;
+  CUmemorytype type{};
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[3] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE,
+                                 CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* to[3] = {&type, &start, &size};
+  return query(3, what, to, at) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE &&
+         at - start + n * sizeof(T) <= size;
+}
+
 // A training batch on the device: the caller's device arrays as they are, or
 // the host arrays in one copy through a pinned image (five copies from pageable
 // memory, each staged by the driver, took half of a step on 4096 samples).
@@ -186,18 +214,25 @@ struct MlpBatch {
 MlpBatch mlp_batch(tp_mlp* a, int B, const float* X, const int* slot, const double* St,
                    const double* Sd, const double* target, int ptr_is_device) {
   a->ensure(B);
-  if (ptr_is_device) return {X, St, Sd, target, slot};
-  if (!a->hbatch) TP_CUDA_TRY(cudaMallocHost(&a->hbatch, (size_t)a->cap * tp_mlp::kBatchBytes));
-  const size_t n = B, nX = n * tp::kMlpIn * sizeof(float), nd = n * sizeof(double);
+  const size_t n = B;
+  if (ptr_is_device && usable_in_place(X, n * tp::kMlpIn) && usable_in_place(slot, n) &&
+      usable_in_place(St, n) && usable_in_place(Sd, n) && usable_in_place(target, n))
+    return {X, St, Sd, target, slot};
+  const size_t nX = n * tp::kMlpIn * sizeof(float), nd = n * sizeof(double);
   const size_t oSt = 0, oSd = nd, oT = 2 * nd, oX = 3 * nd, oS = oX + nX;
-  char* h = a->hbatch;
-  std::memcpy(h + oSt, St, nd);
-  std::memcpy(h + oSd, Sd, nd);
-  std::memcpy(h + oT, target, nd);
-  std::memcpy(h + oX, X, nX);
-  std::memcpy(h + oS, slot, n * sizeof(int));
-  TP_CUDA_TRY(cudaMemcpyAsync(a->batch, h, n * tp_mlp::kBatchBytes, cudaMemcpyHostToDevice, a->s));
+  const struct {
+    size_t at, bytes;
+    const void* from;
+  } part[5] = {{oSt, nd, St}, {oSd, nd, Sd}, {oT, nd, target}, {oX, nX, X}, {oS, n * sizeof(int), slot}};
   char* d = a->batch;
+  if (ptr_is_device) {
+    for (const auto& q : part)
+      TP_CUDA_TRY(cudaMemcpyAsync(d + q.at, q.from, q.bytes, cudaMemcpyDeviceToDevice, a->s));
+  } else {
+    if (!a->hbatch) TP_CUDA_TRY(cudaMallocHost(&a->hbatch, (size_t)a->cap * tp_mlp::kBatchBytes));
+    for (const auto& q : part) std::memcpy(a->hbatch + q.at, q.from, q.bytes);
+    TP_CUDA_TRY(cudaMemcpyAsync(d, a->hbatch, n * tp_mlp::kBatchBytes, cudaMemcpyHostToDevice, a->s));
+  }
   return {reinterpret_cast<float*>(d + oX), reinterpret_cast<double*>(d + oSt),
           reinterpret_cast<double*>(d + oSd), reinterpret_cast<double*>(d + oT),
           reinterpret_cast<int*>(d + oS)};
@@ -576,14 +611,12 @@ int tp_spmv(tp_ctx* c, const double* x_p, const double* x_T, double* y_p, double
   TP_API_BEGIN
   cudaStream_t s = c->s;
   const size_t n = c->N;
-  // device vectors are read and written in place unless an output overlaps an
-  // input (the four copies took a third of the call at 442 k cells)
-  const double* in[2] = {x_p, x_T};
-  double* out[2] = {y_p, y_T};
-  bool overlap = false;
-  for (const double* a : in)
-    for (const double* b : out) overlap = overlap || (a < b + n && b < a + n);
-  if (ptr_is_device && !overlap) {
+  // device vectors are read and written in place unless an output overlaps
+  // another vector (the four copies took a third of the call at 442 k cells)
+  const auto apart = [n](const double* a, const double* b) { return a + n <= b || b + n <= a; };
+  if (ptr_is_device && apart(x_p, y_p) && apart(x_p, y_T) && apart(x_T, y_p) && apart(x_T, y_T) &&
+      apart(y_p, y_T) && usable_in_place(x_p, n) && usable_in_place(x_T, n) &&
+      usable_in_place(y_p, n) && usable_in_place(y_T, n)) {
     tp::launch_block_spmv(c->N, c->rowptr, c->col, c->bval, x_p, x_T, y_p, y_T, nullptr, s);
     TP_CUDA_TRY(cudaStreamSynchronize(s));
     return TP_OK;
