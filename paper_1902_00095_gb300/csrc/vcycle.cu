@@ -14,6 +14,8 @@
 // the vectors the previous kernels wrote after it. The first kernel of a
 // V-cycle (level 0 pre-smoothing) waits first: the kernel before it may be a
 // setup kernel that wrote those operators.
+#include <type_traits>
+
 #include "amg.cuh"
 
 namespace tp {
@@ -180,6 +182,32 @@ __global__ void __launch_bounds__(256) k_jacobi2z(int n, const int* __restrict__
   if (valid && lane == 0) x[row] = d * bi + d * (bi - acc);
 }
 
+// Matrix entries of the sliced-ELL and ELL sweeps. ONCE: loaded past L1, which
+// then holds more of the gathered vector; for levels whose sweep streams more
+// than L2 holds (`streams`), since a line loaded this way is also the first to
+// leave L2 and a smaller level is read from there again by the next sweep
+// (layered 256x256x64, A_pp level 1, 488 MB: FP64 sweep 94 -> 85 us, residual
+// 89 -> 80, FP32 sweep 60 -> 54; with every level loaded so the channel
+// 128x128x64 solve took 19.3 ms against 18.4).
+template <bool ONCE, class T>
+__device__ __forceinline__ T ld_entry(const T* p) {
+  if constexpr (!ONCE) {
+    return __ldg(p);
+  } else if constexpr (sizeof(T) == 8) {
+    double v;
+    asm("ld.global.nc.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+  } else if constexpr (std::is_same_v<T, float>) {
+    float v;
+    asm("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+  } else {
+    int v;
+    asm("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+  }
+}
+
 // column of slot k of row `row` in an ELL copy by grid direction (offsets
 // -nxy, -nx, -1, 0, +1, +nx, +nxy), clamped to [0, n): an absent neighbour's
 // slot holds 0, so any column in range adds an exact zero
@@ -193,7 +221,7 @@ __device__ __forceinline__ int stencil_col(int k, int row, int n, int nx, int nx
 // ELL forms (slot-major, one thread per row, coalesced over rows); a row's
 // slots are held in registers, loaded before the dependency wait. ecol null:
 // the slots are the grid directions of an nx x ny x nz grid (nxy = nx ny)
-template <class TV>
+template <class TV, bool ONCE>
 struct EllRow {
   int c[kEllMaxW];
   TV v[kEllMaxW];
@@ -206,8 +234,8 @@ struct EllRow {
       v[k] = TV(0);
       if (k < w) {
         const long long q = (long long)k * n + row;
-        c[k] = ecol ? ecol[q] : stencil_col(k, row, n, nx, nxy);
-        v[k] = eval[q];
+        c[k] = ecol ? ld_entry<ONCE>(ecol + q) : stencil_col(k, row, n, nx, nxy);
+        v[k] = ld_entry<ONCE>(eval + q);
       }
     }
   }
@@ -222,7 +250,7 @@ struct EllRow {
   }
 };
 
-template <class TV, class TB, class TO>
+template <bool ONCE, class TV, class TB, class TO>
 __global__ void __launch_bounds__(256) k_jacobi_ell(int n, int w, const int* __restrict__ ecol, int snx, int snxy,
                                                     const TV* __restrict__ eval,
                                                     const TV* __restrict__ dinv,
@@ -230,7 +258,7 @@ __global__ void __launch_bounds__(256) k_jacobi_ell(int n, int w, const int* __r
                                                     const TV* __restrict__ xin,
                                                     TO* __restrict__ xout) {
   const int row = blockIdx.x * blockDim.x + threadIdx.x;
-  EllRow<TV> a;
+  EllRow<TV, ONCE> a;
   TV di = TV(0);
   if (row < n) {
     a.load(n, w, ecol, eval, row, snx, snxy);
@@ -244,14 +272,14 @@ __global__ void __launch_bounds__(256) k_jacobi_ell(int n, int w, const int* __r
   xout[row] = (TO)(xi + di * (bi - ax));
 }
 
-template <class TV, class TB>
+template <bool ONCE, class TV, class TB>
 __global__ void __launch_bounds__(256) k_residual_ell(int n, int w, const int* __restrict__ ecol, int snx, int snxy,
                                                       const TV* __restrict__ eval,
                                                       const TB* __restrict__ b,
                                                       const TV* __restrict__ x,
                                                       TV* __restrict__ r) {
   const int row = blockIdx.x * blockDim.x + threadIdx.x;
-  EllRow<TV> a;
+  EllRow<TV, ONCE> a;
   if (row < n) a.load(n, w, ecol, eval, row, snx, snxy);
   pdl_wait();
   pdl_trigger();
@@ -260,7 +288,7 @@ __global__ void __launch_bounds__(256) k_residual_ell(int n, int w, const int* _
   r[row] = bi - a.dot(w, x);
 }
 
-template <class TV, class TB>
+template <bool ONCE, class TV, class TB>
 __global__ void __launch_bounds__(256) k_jacobi2z_ell(int n, int w, const int* __restrict__ ecol,
                                                       int snx, int snxy,
                                                       const TV* __restrict__ eval,
@@ -269,7 +297,7 @@ __global__ void __launch_bounds__(256) k_jacobi2z_ell(int n, int w, const int* _
                                                       const TV* __restrict__ y,
                                                       TV* __restrict__ x) {
   const int row = blockIdx.x * blockDim.x + threadIdx.x;
-  EllRow<TV> a;
+  EllRow<TV, ONCE> a;
   TV d = TV(0);
   if (row < n) {
     a.load(n, w, ecol, eval, row, snx, snxy);
@@ -561,7 +589,7 @@ __global__ void __launch_bounds__(kLineThreads) k_line_block(
 // padding; a row's sum runs over its entries in CSR order. The row of each
 // slot, the slice extent and the first K entries are loaded before the
 // dependency wait.
-template <class TV>
+template <class TV, bool ONCE>
 struct SellRow {
   static constexpr int K = sizeof(TV) >= 8 ? 4 : 8;
   int row = -1, q0 = 0, w = 0;
@@ -582,8 +610,8 @@ struct SellRow {
       c[k] = 0;
       v[k] = TV(0);
       if (k < w) {
-        c[k] = col[q0 + 32 * k];
-        v[k] = val[q0 + 32 * k];
+        c[k] = ld_entry<ONCE>(col + q0 + 32 * k);
+        v[k] = ld_entry<ONCE>(val + q0 + 32 * k);
       }
     }
   }
@@ -616,8 +644,8 @@ struct SellRow {
           cn[j] = 0;
           vn[j] = TV(0);
           if (k < w) {
-            cn[j] = col[q0 + 32 * k];
-            vn[j] = val[q0 + 32 * k];
+            cn[j] = ld_entry<ONCE>(col + q0 + 32 * k);
+            vn[j] = ld_entry<ONCE>(val + q0 + 32 * k);
           }
         }
 #pragma unroll
@@ -633,13 +661,14 @@ struct SellRow {
 #pragma unroll
       for (int k = 0; k < K; ++k)
         if (k < w) acc += v[k] * (TV)x[c[k]];
-      for (int k = K; k < w; ++k) acc += val[q0 + 32 * k] * (TV)x[col[q0 + 32 * k]];
+      for (int k = K; k < w; ++k)
+        acc += ld_entry<ONCE>(val + q0 + 32 * k) * (TV)x[ld_entry<ONCE>(col + q0 + 32 * k)];
     }
     return acc;
   }
 };
 
-template <class TV, class TB, class TO>
+template <bool ONCE, class TV, class TB, class TO>
 __global__ void __launch_bounds__(256) k_sell_jacobi(int nslots, const int* __restrict__ ptr,
                                                      const int* __restrict__ perm,
                                                      const int* __restrict__ col,
@@ -649,7 +678,7 @@ __global__ void __launch_bounds__(256) k_sell_jacobi(int nslots, const int* __re
                                                      const TV* __restrict__ xin,
                                                      TO* __restrict__ xout) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  SellRow<TV> a;
+  SellRow<TV, ONCE> a;
   a.load(nslots, ptr, perm, col, val, t);
   const TV di = a.row >= 0 ? dinv[a.row] : TV(0);
   pdl_wait();
@@ -660,7 +689,7 @@ __global__ void __launch_bounds__(256) k_sell_jacobi(int nslots, const int* __re
   xout[a.row] = (TO)(xi + di * (bi - ax));
 }
 
-template <class TV, class TB>
+template <bool ONCE, class TV, class TB>
 __global__ void __launch_bounds__(256) k_sell_residual(int nslots, const int* __restrict__ ptr,
                                                        const int* __restrict__ perm,
                                                        const int* __restrict__ col,
@@ -669,7 +698,7 @@ __global__ void __launch_bounds__(256) k_sell_residual(int nslots, const int* __
                                                        const TV* __restrict__ x,
                                                        TV* __restrict__ r) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  SellRow<TV> a;
+  SellRow<TV, ONCE> a;
   a.load(nslots, ptr, perm, col, val, t);
   pdl_wait();
   pdl_trigger();
@@ -682,7 +711,7 @@ __global__ void __launch_bounds__(256) k_sell_residual(int nslots, const int* __
 // (with the row sum of the other sweeps: a loop of its own without the FP64
 // prefetch took 101 us a launch on A_pp's sliced levels of the layered
 // 256x256x64 system, this 78)
-template <class TV, class TB>
+template <bool ONCE, class TV, class TB>
 __global__ void __launch_bounds__(256) k_sell_jacobi2z(int nslots, const int* __restrict__ ptr,
                                                        const int* __restrict__ perm,
                                                        const int* __restrict__ col,
@@ -692,7 +721,7 @@ __global__ void __launch_bounds__(256) k_sell_jacobi2z(int nslots, const int* __
                                                        const TV* __restrict__ y,
                                                        TV* __restrict__ x) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  SellRow<TV> a;
+  SellRow<TV, ONCE> a;
   a.load(nslots, ptr, perm, col, val, t);
   const TV d = a.row >= 0 ? dinv[a.row] : TV(0);
   pdl_wait();
@@ -816,53 +845,6 @@ struct Vals<float> {
 // `final_out` (type TO) when non-null, else to one of the level's work
 // vectors, whose address is returned.
 // level operations: ELL when the level has an ELL copy, CSR otherwise
-template <class TV, class TB, class TO>
-void level_sweep(const Level& v, const TV* dinv, const TB* b, const TV* xin, TO* xout,
-                 cudaStream_t s) {
-  if (v.sell_slices > 0) {
-    const int nslots = v.sell_slices * 32;
-    launch_pdl(k_sell_jacobi<TV, TB, TO>, grid_for(nslots), kBlock, s, nslots, v.sell_ptr,
-               v.sell_perm, v.sell_col, Vals<TV>::S(v), dinv, b, xin, xout);
-  } else if (v.ell_w > 0) {
-    launch_pdl(k_jacobi_ell<TV, TB, TO>, grid_for(v.A.n), kBlock, s, v.A.n, v.ell_w, v.ell_col,
-               v.ell_nx, v.ell_nxy, Vals<TV>::E(v), dinv, b, xin, xout);
-  } else {
-    jacobi<TV, TB, TO>(v.lanes_A, v.A, Vals<TV>::A(v), dinv, b, xin, xout, s);
-  }
-}
-
-template <class TV, class TB>
-void level_residual(const Level& v, const TB* b, const TV* x, TV* r, cudaStream_t s) {
-  if (v.sell_slices > 0) {
-    const int nslots = v.sell_slices * 32;
-    launch_pdl(k_sell_residual<TV, TB>, grid_for(nslots), kBlock, s, nslots, v.sell_ptr,
-               v.sell_perm, v.sell_col, Vals<TV>::S(v), b, x, r);
-  } else if (v.ell_w > 0) {
-    launch_pdl(k_residual_ell<TV, TB>, grid_for(v.A.n), kBlock, s, v.A.n, v.ell_w, v.ell_col,
-               v.ell_nx, v.ell_nxy, Vals<TV>::E(v), b, x, r);
-  } else {
-    residual<TV, TB>(v.lanes_A, v.A, Vals<TV>::A(v), b, x, r, s);
-  }
-}
-
-// y: work vector of the level (holds d b); first: the sweeps open a V-cycle
-// (the first kernel waits before any read)
-template <class TV, class TB>
-void level_two_sweeps_from_zero(const Level& v, const TV* dinv, const TB* b, TV* y, TV* x,
-                                int first, cudaStream_t s, bool y_ready = false) {
-  if (!y_ready)
-    launch_pdl(k_scale_db<TV, TB>, grid_for(v.A.n), kBlock, s, v.A.n, dinv, b, y, first);
-  if (v.sell_slices > 0) {
-    const int nslots = v.sell_slices * 32;
-    launch_pdl(k_sell_jacobi2z<TV, TB>, grid_for(nslots), kBlock, s, nslots, v.sell_ptr,
-               v.sell_perm, v.sell_col, Vals<TV>::S(v), dinv, b, (const TV*)y, x);
-  } else if (v.ell_w > 0) {
-    launch_pdl(k_jacobi2z_ell<TV, TB>, grid_for(v.A.n), kBlock, s, v.A.n, v.ell_w, v.ell_col,
-               v.ell_nx, v.ell_nxy, Vals<TV>::E(v), dinv, b, (const TV*)y, x);
-  } else {
-    jacobi2z<TV, TB>(v.lanes_A, v.A, Vals<TV>::A(v), dinv, b, y, x, s);
-  }
-}
 
 // algorithmic bytes of one sweep x_out = x_in + dinv (b - A x_in)
 template <class TV, class TB, class TO>
@@ -873,6 +855,97 @@ double sweep_bytes(const Level& v) {
   const double amat = v.ell_nxy > 0 ? (double)A.n * v.ell_w * sizeof(TV)
                                     : (double)A.nnz * (sizeof(TV) + sizeof(int)) + 4.0 * (A.n + 1);
   return amat + (double)A.n * (2 * sizeof(TV) + sizeof(TB) + sizeof(TO));
+}
+
+// Whether a sweep over the level leaves nothing of its matrix in L2 for the
+// next one: 1.4 times the 129 MB of L2. On the layered 256x256x64 levels the
+// loads past L1 gain 5-12 % from 185 MB on (FP32 S~ level 2, 41.0 -> 39.5 us),
+// 0-2 % at 110-174 MB (A_pp level 2) and cost 1-4 % below that.
+constexpr double kStreamBytes = 180e6;
+
+template <class TV>
+bool streams(const Level& v) {
+  return sweep_bytes<TV, TV, TV>(v) > kStreamBytes;
+}
+
+// Threads per block of the sliced-ELL kernels. Rows are sorted by length over
+// 256, so a block of 256 in FP64 holds its registers until its longest rows
+// are done; blocks of 128 turn over sooner (A_pp level 1 sweep 92 -> 85 us,
+// level 2 48 -> 46; of 64: 87, 47). FP32 sweeps have no FP64 pipe to fill and
+// gain more from the rows that share vector lines in one L1 (256: 54 us, 512:
+// 55, 64: 63).
+template <class TV>
+constexpr int kSellBlock = sizeof(TV) >= 8 ? 128 : 256;
+
+template <bool ONCE, class TV, class TB, class TO>
+void stored_sweep(const Level& v, const TV* dinv, const TB* b, const TV* xin, TO* xout,
+                  cudaStream_t s) {
+  const int nslots = v.sell_slices * 32;
+  if (v.sell_slices > 0)
+    launch_pdl(k_sell_jacobi<ONCE, TV, TB, TO>, grid_for(nslots, kSellBlock<TV>), kSellBlock<TV>,
+               s, nslots, v.sell_ptr, v.sell_perm, v.sell_col, Vals<TV>::S(v), dinv, b, xin, xout);
+  else
+    launch_pdl(k_jacobi_ell<ONCE, TV, TB, TO>, grid_for(v.A.n), kBlock, s, v.A.n, v.ell_w,
+               v.ell_col, v.ell_nx, v.ell_nxy, Vals<TV>::E(v), dinv, b, xin, xout);
+}
+
+template <bool ONCE, class TV, class TB>
+void stored_residual(const Level& v, const TB* b, const TV* x, TV* r, cudaStream_t s) {
+  const int nslots = v.sell_slices * 32;
+  if (v.sell_slices > 0)
+    launch_pdl(k_sell_residual<ONCE, TV, TB>, grid_for(nslots, kSellBlock<TV>), kSellBlock<TV>, s,
+               nslots, v.sell_ptr, v.sell_perm, v.sell_col, Vals<TV>::S(v), b, x, r);
+  else
+    launch_pdl(k_residual_ell<ONCE, TV, TB>, grid_for(v.A.n), kBlock, s, v.A.n, v.ell_w,
+               v.ell_col, v.ell_nx, v.ell_nxy, Vals<TV>::E(v), b, x, r);
+}
+
+template <bool ONCE, class TV, class TB>
+void stored_two_sweeps(const Level& v, const TV* dinv, const TB* b, const TV* y, TV* x,
+                       cudaStream_t s) {
+  const int nslots = v.sell_slices * 32;
+  if (v.sell_slices > 0)
+    launch_pdl(k_sell_jacobi2z<ONCE, TV, TB>, grid_for(nslots, kSellBlock<TV>), kSellBlock<TV>, s,
+               nslots, v.sell_ptr, v.sell_perm, v.sell_col, Vals<TV>::S(v), dinv, b, y, x);
+  else
+    launch_pdl(k_jacobi2z_ell<ONCE, TV, TB>, grid_for(v.A.n), kBlock, s, v.A.n, v.ell_w,
+               v.ell_col, v.ell_nx, v.ell_nxy, Vals<TV>::E(v), dinv, b, y, x);
+}
+
+template <class TV, class TB, class TO>
+void level_sweep(const Level& v, const TV* dinv, const TB* b, const TV* xin, TO* xout,
+                 cudaStream_t s) {
+  if (v.sell_slices == 0 && v.ell_w == 0)
+    jacobi<TV, TB, TO>(v.lanes_A, v.A, Vals<TV>::A(v), dinv, b, xin, xout, s);
+  else if (streams<TV>(v))
+    stored_sweep<true, TV, TB, TO>(v, dinv, b, xin, xout, s);
+  else
+    stored_sweep<false, TV, TB, TO>(v, dinv, b, xin, xout, s);
+}
+
+template <class TV, class TB>
+void level_residual(const Level& v, const TB* b, const TV* x, TV* r, cudaStream_t s) {
+  if (v.sell_slices == 0 && v.ell_w == 0)
+    residual<TV, TB>(v.lanes_A, v.A, Vals<TV>::A(v), b, x, r, s);
+  else if (streams<TV>(v))
+    stored_residual<true, TV, TB>(v, b, x, r, s);
+  else
+    stored_residual<false, TV, TB>(v, b, x, r, s);
+}
+
+// y: work vector of the level (holds d b); first: the sweeps open a V-cycle
+// (the first kernel waits before any read)
+template <class TV, class TB>
+void level_two_sweeps_from_zero(const Level& v, const TV* dinv, const TB* b, TV* y, TV* x,
+                                int first, cudaStream_t s, bool y_ready = false) {
+  if (!y_ready)
+    launch_pdl(k_scale_db<TV, TB>, grid_for(v.A.n), kBlock, s, v.A.n, dinv, b, y, first);
+  if (v.sell_slices == 0 && v.ell_w == 0)
+    jacobi2z<TV, TB>(v.lanes_A, v.A, Vals<TV>::A(v), dinv, b, y, x, s);
+  else if (streams<TV>(v))
+    stored_two_sweeps<true, TV, TB>(v, dinv, b, y, x, s);
+  else
+    stored_two_sweeps<false, TV, TB>(v, dinv, b, y, x, s);
 }
 
 template <class TV, class TB, class TO>
