@@ -163,10 +163,10 @@ class ClockSampler:
 
 
 PROBE_NAMES = {0: "k_jacobi_ell (finest A_pp level, l1-Jacobi sweep, ELL)",
-               1: "k_line_sweep (finest S~ level, vertical-line step)",
+               1: "k_line_block (finest S~ level, vertical-line step)",
                2: "k_block_spmv (2x2 block-CSR SpMV, FP64)",
                3: "k_jacobi (A_pp level 1, l1-Jacobi sweep, CSR)"}
-# class 3 when level 1 keeps a sliced-ELL copy (levels of a full wave of
+# class 3 when level 1 keeps a sliced-ELL copy (levels of half a wave of
 # resident threads or more)
 PROBE_NAME_SLICED = "k_sell_jacobi (A_pp level 1, l1-Jacobi sweep, sliced ELL)"
 

@@ -936,7 +936,7 @@ __global__ void k_to_bf16(long long n, const double* __restrict__ a,
 // Correctly rounded operations in the oracle's order (no FMA contraction).
 // Twisted factorisation of each column's tridiagonal part (diagonal d_k,
 // lower l_k, upper u_k; layer k of column c is cell c + nxy k), so that two
-// threads can solve a column from both ends at once (k_line_sweep). With
+// threads can solve a column from both ends at once (k_line_block). With
 // mid = nz / 2: the top rows k < mid are eliminated downwards (m_k = d_k -
 // l_k cp_{k-1}, cp_k = u_k / m_k), the bottom rows k > mid upwards (q_k =
 // d_k - u_k cq_{k+1}, cq_k = l_k / q_k), and the middle row takes both sides

@@ -204,7 +204,7 @@ bool usable_in_place(const T* p, size_t n) {
 
 // A training batch on the device: the caller's device arrays as they are, or
 // the host arrays in one copy through a pinned image (five copies from pageable
-// memory, each staged by the driver, took half of a step on 4096 samples).
+// memory, each staged by the runtime, took half of a step on 4096 samples).
 struct MlpBatch {
   const float* X;
   const double *St, *Sd, *target;
