@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <thread>
 #include <cuda.h>
+#include "mlp_stage.cuh"
 #include "solver.cuh"
 
 using tp::Error;
@@ -145,32 +146,11 @@ struct tp_mlp {
   bool own_stream = false;
   tp::Pool pool;
   tp::MlpDev m;
-  tp::Pool stage;  // device copies of host inputs
-  int cap = 0;
-  float* X = nullptr;
-  char* batch = nullptr;    // device copy of a training batch, kBatchBytes per sample
-  char* hbatch = nullptr;   // pinned image of it
-  float* O = nullptr;
-  float* partials = nullptr;
+  tp::MlpStage stage;      // batches
   double* host = nullptr;  // pinned [kMlpPartial]
-  static constexpr size_t kBatchBytes = sizeof(float) * tp::kMlpIn + 3 * sizeof(double) + sizeof(int);
   ~tp_mlp() {
-    stage.release();
-    pool.release();
     if (host) cudaFreeHost(host);
-    if (hbatch) cudaFreeHost(hbatch);
     if (own_stream && s) cudaStreamDestroy(s);
-  }
-  void ensure(int n) {
-    if (n <= cap) return;
-    stage.release();
-    cap = n;
-    X = stage.alloc<float>((size_t)n * tp::kMlpIn);
-    batch = stage.alloc<char>((size_t)n * kBatchBytes);
-    if (hbatch) cudaFreeHost(hbatch);
-    hbatch = nullptr;
-    O = stage.alloc<float>((size_t)n * tp::kMlpOut);
-    partials = stage.alloc<float>((size_t)((n + 15) / 16) * tp::kMlpPartial);
   }
 };
 
@@ -213,7 +193,7 @@ struct MlpBatch {
 
 MlpBatch mlp_batch(tp_mlp* a, int B, const float* X, const int* slot, const double* St,
                    const double* Sd, const double* target, int ptr_is_device) {
-  a->ensure(B);
+  a->stage.ensure(B);
   const size_t n = B;
   if (ptr_is_device && usable_in_place(X, n * tp::kMlpIn) && usable_in_place(slot, n) &&
       usable_in_place(St, n) && usable_in_place(Sd, n) && usable_in_place(target, n))
@@ -224,14 +204,14 @@ MlpBatch mlp_batch(tp_mlp* a, int B, const float* X, const int* slot, const doub
     size_t at, bytes;
     const void* from;
   } part[5] = {{oSt, nd, St}, {oSd, nd, Sd}, {oT, nd, target}, {oX, nX, X}, {oS, n * sizeof(int), slot}};
-  char* d = a->batch;
+  char* d = a->stage.batch;
   if (ptr_is_device) {
     for (const auto& q : part)
       TP_CUDA_TRY(cudaMemcpyAsync(d + q.at, q.from, q.bytes, cudaMemcpyDeviceToDevice, a->s));
   } else {
-    if (!a->hbatch) TP_CUDA_TRY(cudaMallocHost(&a->hbatch, (size_t)a->cap * tp_mlp::kBatchBytes));
-    for (const auto& q : part) std::memcpy(a->hbatch + q.at, q.from, q.bytes);
-    TP_CUDA_TRY(cudaMemcpyAsync(d, a->hbatch, n * tp_mlp::kBatchBytes, cudaMemcpyHostToDevice, a->s));
+    char* h = a->stage.host_image();
+    for (const auto& q : part) std::memcpy(h + q.at, q.from, q.bytes);
+    TP_CUDA_TRY(cudaMemcpyAsync(d, h, n * tp::MlpStage::kBatchBytes, cudaMemcpyHostToDevice, a->s));
   }
   return {reinterpret_cast<float*>(d + oX), reinterpret_cast<double*>(d + oSt),
           reinterpret_cast<double*>(d + oSd), reinterpret_cast<double*>(d + oT),
@@ -919,14 +899,14 @@ int tp_mlp_forward(tp_mlp* a, int n, const float* X, float* O, int ptr_is_device
   const float* Xd = X;
   float* Od = O;
   if (!ptr_is_device) {
-    a->ensure(n);
-    TP_CUDA_TRY(cudaMemcpyAsync(a->X, X, sizeof(float) * n * tp::kMlpIn, cudaMemcpyHostToDevice, a->s));
-    Xd = a->X;
-    Od = a->O;
+    a->stage.ensure(n);
+    TP_CUDA_TRY(cudaMemcpyAsync(a->stage.X, X, sizeof(float) * n * tp::kMlpIn, cudaMemcpyHostToDevice, a->s));
+    Xd = a->stage.X;
+    Od = a->stage.O;
   }
   tp::mlp_forward(a->m, n, Xd, Od, a->s);
   if (!ptr_is_device)
-    TP_CUDA_TRY(cudaMemcpyAsync(O, a->O, sizeof(float) * n * tp::kMlpOut, cudaMemcpyDeviceToHost, a->s));
+    TP_CUDA_TRY(cudaMemcpyAsync(O, a->stage.O, sizeof(float) * n * tp::kMlpOut, cudaMemcpyDeviceToHost, a->s));
   TP_CUDA_TRY(cudaStreamSynchronize(a->s));
   return TP_OK;
   TP_API_END
@@ -938,7 +918,7 @@ int tp_mlp_gradient(tp_mlp* a, int B, const float* X, const int* slot, const dou
   if (!a || B < 1 || !X || !slot || !St || !Sd || !target) return TP_EINVAL;
   TP_API_BEGIN
   const MlpBatch t = mlp_batch(a, B, X, slot, St, Sd, target, ptr_is_device);
-  tp::mlp_gradient(a->m, B, t.X, t.slot, t.St, t.Sd, t.target, a->partials, a->m.grad, a->s);
+  tp::mlp_gradient(a->m, B, t.X, t.slot, t.St, t.Sd, t.target, a->stage.partials, a->m.grad, a->s);
   std::vector<float> f(tp::kMlpPartial);
   TP_CUDA_TRY(cudaMemcpyAsync(f.data(), a->m.grad, sizeof(float) * tp::kMlpPartial,
                               cudaMemcpyDeviceToHost, a->s));
@@ -956,7 +936,7 @@ int tp_mlp_train_step(tp_mlp* a, int B, const float* X, const int* slot, const d
   if (!a || B < 1 || !X || !slot || !St || !Sd || !target || !(lr > 0.0)) return TP_EINVAL;
   TP_API_BEGIN
   const MlpBatch t = mlp_batch(a, B, X, slot, St, Sd, target, ptr_is_device);
-  tp::mlp_train_step(a->m, B, t.X, t.slot, t.St, t.Sd, t.target, a->partials, a->m.grad,
+  tp::mlp_train_step(a->m, B, t.X, t.slot, t.St, t.Sd, t.target, a->stage.partials, a->m.grad,
                      (float)lr, a->s);
   float* l = reinterpret_cast<float*>(a->host);
   TP_CUDA_TRY(cudaMemcpyAsync(l, a->m.grad + tp::kMlpParams, sizeof(float), cudaMemcpyDeviceToHost, a->s));

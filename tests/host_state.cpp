@@ -1,0 +1,102 @@
+// Host logic of the library's headers against a fake CUDA runtime (no GPU):
+// compiled and run by test_host_state.py, one check per argument. A check that
+// fails prints its line and exits with 1.
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+
+#include "mlp_stage.cuh"
+
+// ---------------------------------------------------------------- fake runtime
+static size_t g_device_limit = ~size_t(0), g_device_used = 0;
+static std::map<char*, size_t> g_device, g_pinned;
+
+extern "C" {
+cudaError_t cudaMalloc(void** p, size_t n) {
+  if (g_device_used + n > g_device_limit) return cudaErrorMemoryAllocation;
+  static char* next = reinterpret_cast<char*>(size_t(1) << 40);  // addresses only
+  *p = next;
+  next += n + 4096;
+  g_device[static_cast<char*>(*p)] = n;
+  g_device_used += n;
+  return cudaSuccess;
+}
+cudaError_t cudaFree(void* p) {
+  if (!p) return cudaSuccess;
+  g_device_used -= g_device.at(static_cast<char*>(p));
+  g_device.erase(static_cast<char*>(p));
+  return cudaSuccess;
+}
+cudaError_t cudaMallocHost(void** p, size_t n) {
+  *p = std::malloc(n);
+  g_pinned[static_cast<char*>(*p)] = n;
+  return cudaSuccess;
+}
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return cudaMallocHost(p, n); }
+cudaError_t cudaFreeHost(void* p) {
+  g_pinned.erase(static_cast<char*>(p));
+  std::free(p);
+  return cudaSuccess;
+}
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+const char* cudaGetErrorString(cudaError_t) { return "fake"; }
+}
+
+#define CHECK(x)                                             \
+  do {                                                       \
+    if (!(x)) {                                              \
+      std::printf("%s:%d: %s\n", __FILE__, __LINE__, #x);    \
+      std::exit(1);                                          \
+    }                                                        \
+  } while (0)
+
+// [p, p + n) lies in one live allocation
+static bool inside(const std::map<char*, size_t>& m, const void* p, size_t n) {
+  const char* c = static_cast<const char*>(p);
+  for (const auto& a : m)
+    if (c >= a.first && c + n <= a.first + a.second) return true;
+  return false;
+}
+
+// a growth of a network's batch buffers that runs out of memory at any of them
+// leaves nothing that a later, smaller batch could run past
+static void mlp_growth() {
+  for (size_t limit = 8u << 20; limit < (1700u << 20); limit += 8u << 20) {
+    tp::MlpStage st;
+    g_device_limit = ~size_t(0);
+    st.ensure(64);
+    st.host_image();
+    g_device_limit = limit;
+    bool failed = false;
+    try {
+      st.ensure(1000000);
+    } catch (const tp::Error& e) {
+      failed = e.code == TP_ENOMEM;
+    }
+    CHECK(failed == (st.cap == 0));
+    g_device_limit = ~size_t(0);
+    const size_t n = 5000;
+    st.ensure((int)n);
+    CHECK(inside(g_device, st.X, n * tp::kMlpIn * sizeof(float)));
+    CHECK(inside(g_device, st.batch, n * tp::MlpStage::kBatchBytes));
+    CHECK(inside(g_device, st.O, n * tp::kMlpOut * sizeof(float)));
+    CHECK(inside(g_device, st.partials, (n + 15) / 16 * tp::kMlpPartial * sizeof(float)));
+    CHECK(inside(g_pinned, st.host_image(), n * tp::MlpStage::kBatchBytes));
+  }
+  CHECK(g_device.empty() && g_pinned.empty());
+}
+
+int main(int, char** argv) {
+  const struct {
+    const char* name;
+    void (*run)();
+  } checks[] = {{"mlp_growth", mlp_growth}};
+  for (const auto& c : checks)
+    if (std::strcmp(argv[1], c.name) == 0) {
+      c.run();
+      return 0;
+    }
+  std::printf("no such check\n");
+  return 1;
+}
