@@ -1129,15 +1129,12 @@ int assemble_device(tp_ctx* c, double dt) {
 }
 
 // the scalar blocks of the assembled matrix on its pattern, and the coupling
-// blocks by grid direction
+// blocks by grid direction where there is memory for them
 void extract_blocks(tp_ctx* c) {
   launch_extract_blocks(c->nnzb, c->bval, c->App, c->ApT, c->ATp, c->ATT, c->s);
   if (c->grid.nx < 2 || c->grid.ny < 2 || c->grid.nz < 2) return;
-  if (!c->ApT_grid) {
-    c->ApT_grid = c->pool.alloc<double>(7 * (size_t)c->N);
-    c->ATp_grid = c->pool.alloc<double>(7 * (size_t)c->N);
-  }
-  launch_coupling_planes(c->grid, c->rowptr, c->bval, c->ApT_grid, c->ATp_grid, c->s);
+  if (c->planes.ensure(c->N))
+    launch_coupling_planes(c->grid, c->rowptr, c->bval, c->planes.ApT, c->planes.ATp, c->s);
 }
 
 // features -> MLP -> corrected S~ with the per-row guard; more than a quarter
@@ -1285,6 +1282,7 @@ void build_device(tp_ctx* c, const tp_precond_opts& o) {
   c->probe_nodes.clear();
   c->probe_set = 0;
   c->built = false;
+  c->planes.refused = false;
   extract_blocks(c);
   launch_equation_scales(c->N, c->dpos, c->App, c->ATT, c->tmpN, c->partials, c->nparts,
                          c->scales, s);

@@ -1112,7 +1112,7 @@ void launch_block_spmv(int N, const int* rowptr, const int* col, const double* b
 }
 
 // out = b - A x for a coupling block: from its planes by grid direction when
-// the context keeps them (every grid extent at least 2), else from CSR
+// the context has them (every grid extent at least 2), else from CSR
 static void rhs_minus(tp_ctx* c, const double* csr, const double* plane, const double* b,
                       const double* x, double* out, cudaStream_t s) {
   const int N = c->N;
@@ -1128,10 +1128,10 @@ void precond_record(tp_ctx* c, cudaStream_t s) {
   Hierarchy& hp = *c->hpp;
   Hierarchy& hs = *c->hS;
   hp.vcycle(s);  // step 1: x_p = V_pp(b_p)
-  rhs_minus(c, c->ATp, c->ATp_grid, c->bT_s, hp.out, hs.in, s);  // step 2
+  rhs_minus(c, c->ATp, c->planes.ATp, c->bT_s, hp.out, hs.in, s);  // step 2
   hs.vcycle(s);  // step 3: d_T = V_S(bt_T)
   if (c->opts.variant == 0) {
-    rhs_minus(c, c->ApT, c->ApT_grid, c->bp_s, hs.out, hp.in, s);  // step 4
+    rhs_minus(c, c->ApT, c->planes.ApT, c->bp_s, hs.out, hp.in, s);  // step 4
     hp.vcycle(s);  // step 5: d_p = V_pp(bt_p)
   }
 }

@@ -4,6 +4,7 @@
 #include "amg.cuh"
 #include "kernels.cuh"
 #include "learned.cuh"
+#include "planes.cuh"
 
 namespace tp {
 struct ColumnLane;  // krylov.cu
@@ -37,9 +38,9 @@ struct tp_ctx {
   double* Sval = nullptr;  // [nnzb]
   double *Rm = nullptr, *Re = nullptr;
   double *App = nullptr, *ApT = nullptr, *ATp = nullptr, *ATT = nullptr;
-  // A_pT and A_Tp by grid direction ([7][N], k_coupling_planes), null when a
-  // grid extent is 1
-  double *ApT_grid = nullptr, *ATp_grid = nullptr;
+  // A_pT and A_Tp by grid direction, null when a grid extent is 1 or there was
+  // no memory for them
+  tp::CouplingPlanes planes;
   double* scales = nullptr;  // [2] equation scales s_m, s_e
   double* ones = nullptr;    // [2] = {1, 1}
   double* fscale = nullptr;  // [2] scaling of the Newton function norm

@@ -7,6 +7,7 @@
 #include <map>
 
 #include "mlp_stage.cuh"
+#include "planes.cuh"
 
 // ---------------------------------------------------------------- fake runtime
 static size_t g_device_limit = ~size_t(0), g_device_used = 0;
@@ -87,11 +88,30 @@ static void mlp_growth() {
   CHECK(g_device.empty() && g_pinned.empty());
 }
 
+// memory for one plane but not for two: neither is there, now and when asked
+// again, and both once there is room after a build
+static void coupling_planes() {
+  const size_t N = 1000001;
+  {
+    tp::CouplingPlanes p;
+    g_device_limit = 7 * N * sizeof(double) + (4u << 20);
+    CHECK(!p.ensure(N) && !p.ApT && !p.ATp);
+    g_device_limit = ~size_t(0);
+    CHECK(!p.ensure(N) && !p.ApT && !p.ATp);
+    p.refused = false;
+    CHECK(p.ensure(N));
+    CHECK(inside(g_device, p.ApT, 7 * N * sizeof(double)));
+    CHECK(inside(g_device, p.ATp, 7 * N * sizeof(double)));
+    CHECK(p.ATp >= p.ApT + 7 * N);
+  }
+  CHECK(g_device.empty());
+}
+
 int main(int, char** argv) {
   const struct {
     const char* name;
     void (*run)();
-  } checks[] = {{"mlp_growth", mlp_growth}};
+  } checks[] = {{"mlp_growth", mlp_growth}, {"coupling_planes", coupling_planes}};
   for (const auto& c : checks)
     if (std::strcmp(argv[1], c.name) == 0) {
       c.run();

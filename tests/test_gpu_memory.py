@@ -1,0 +1,61 @@
+"""Calls on a device whose memory is nearly all taken give the results of the
+same calls with memory to spare: what is kept for speed alone is left out or
+given back."""
+import gc
+
+import numpy as np
+import pytest
+
+from synthetic import make_problem
+from synthetic.recipes import perturbed_state
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+thermo = pytest.importorskip("paper_1902_00095_gb300.thermo")
+
+
+class Taken:
+    """Takes device memory until about `leave` bytes are free."""
+
+    def __init__(self, leave):
+        self.leave = leave
+
+    def __enter__(self):
+        torch.cuda.synchronize()
+        self.held = []
+        for block in (1 << 33, 1 << 28, 12 << 20):
+            while torch.cuda.mem_get_info()[0] >= self.leave + block:
+                self.held.append(torch.empty(block, dtype=torch.uint8, device="cuda"))
+        return self
+
+    def __exit__(self, *exc):
+        self.held = None
+        gc.collect()
+        torch.cuda.empty_cache()
+
+
+def solver(shape, seed=4):
+    prob = make_problem("tiny", shape=shape, seed=seed)
+    p, T = perturbed_state(prob, seed=seed + 1)
+    s = thermo.Solver.from_problem(prob)
+    s.assemble(p, T, prob["p_n"], prob["T_n"], prob["dt"])
+    return s
+
+
+# 800,000 cells: 45 MB a plane
+def test_no_room_for_coupling_planes():
+    shape = (100, 100, 80)
+    ref = solver(shape)
+    scales = ref.export_system()[4]
+    ref.build(variant=1)
+    x = ref.solve(rtol=1e-8)
+    ref.close()
+    s = solver(shape)
+    for leave in (60 << 20, 16 << 20):  # one plane and not two; none
+        with Taken(leave):
+            assert np.array_equal(s.export_system()[4], scales)
+    s.build(variant=1)
+    y = s.solve(rtol=1e-8)
+    assert y[2]["iters"] == x[2]["iters"] and np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1])
+    s.close()

@@ -27,7 +27,7 @@ def checks(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("name", ["mlp_growth"])
+@pytest.mark.parametrize("name", ["mlp_growth", "coupling_planes"])
 def test_host_state(checks, name):
     r = subprocess.run([checks, name], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
