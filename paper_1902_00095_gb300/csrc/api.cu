@@ -5,7 +5,7 @@
 #include <cstring>
 #include <algorithm>
 #include <thread>
-#include <cuda.h>
+#include "in_place.cuh"
 #include "mlp_stage.cuh"
 #include "solver.cuh"
 
@@ -143,6 +143,7 @@ struct tp_amg {
 
 struct tp_mlp {
   cudaStream_t s = nullptr;
+  int device = 0;
   bool own_stream = false;
   tp::Pool pool;
   tp::MlpDev m;
@@ -155,31 +156,17 @@ struct tp_mlp {
 };
 
 namespace {
-// Whether a kernel may use the caller's array where it lies: device memory,
-// aligned to its type, `n` elements inside one allocation. A copy accepts any
-// address and reports what it cannot reach, so everything else goes through one.
 template <class T>
-bool usable_in_place(const T* p, size_t n) {
-  using Query = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
-  static const Query query = [] {
+bool usable_in_place(int device, const T* p, size_t n) {
+  static const tp::PointerQuery query = [] {
     void* f = nullptr;
     cudaDriverEntryPointQueryResult r;
     if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault,
                                          &r) != cudaSuccess)
       cudaGetLastError();
-    return reinterpret_cast<Query>(f);
+    return reinterpret_cast<tp::PointerQuery>(f);
   }();
-  const auto at = reinterpret_cast<uintptr_t>(p);
-  if (!query || at % alignof(T)) return false;
-  CUmemorytype type{};
-  CUdeviceptr start = 0;
-  size_t size = 0;
-  CUpointer_attribute what[3] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE,
-                                 CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
-                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE};
-  void* to[3] = {&type, &start, &size};
-  return query(3, what, to, at) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE &&
-         at - start + n * sizeof(T) <= size;
+  return tp::usable_in_place(query, device, p, n);
 }
 
 // A training batch on the device: the caller's device arrays as they are, or
@@ -195,8 +182,10 @@ MlpBatch mlp_batch(tp_mlp* a, int B, const float* X, const int* slot, const doub
                    const double* Sd, const double* target, int ptr_is_device) {
   a->stage.ensure(B);
   const size_t n = B;
-  if (ptr_is_device && usable_in_place(X, n * tp::kMlpIn) && usable_in_place(slot, n) &&
-      usable_in_place(St, n) && usable_in_place(Sd, n) && usable_in_place(target, n))
+  const int dev = a->device;
+  if (ptr_is_device && usable_in_place(dev, X, n * tp::kMlpIn) && usable_in_place(dev, slot, n) &&
+      usable_in_place(dev, St, n) && usable_in_place(dev, Sd, n) &&
+      usable_in_place(dev, target, n))
     return {X, St, Sd, target, slot};
   const size_t nX = n * tp::kMlpIn * sizeof(float), nd = n * sizeof(double);
   const size_t oSt = 0, oSd = nd, oT = 2 * nd, oX = 3 * nd, oS = oX + nX;
@@ -595,8 +584,9 @@ int tp_spmv(tp_ctx* c, const double* x_p, const double* x_T, double* y_p, double
   // another vector (the four copies took a third of the call at 442 k cells)
   const auto apart = [n](const double* a, const double* b) { return a + n <= b || b + n <= a; };
   if (ptr_is_device && apart(x_p, y_p) && apart(x_p, y_T) && apart(x_T, y_p) && apart(x_T, y_T) &&
-      apart(y_p, y_T) && usable_in_place(x_p, n) && usable_in_place(x_T, n) &&
-      usable_in_place(y_p, n) && usable_in_place(y_T, n)) {
+      apart(y_p, y_T) && usable_in_place(c->device, x_p, n) &&
+      usable_in_place(c->device, x_T, n) && usable_in_place(c->device, y_p, n) &&
+      usable_in_place(c->device, y_T, n)) {
     tp::launch_block_spmv(c->N, c->rowptr, c->col, c->bval, x_p, x_T, y_p, y_T, nullptr, s);
     TP_CUDA_TRY(cudaStreamSynchronize(s));
     return TP_OK;
@@ -816,6 +806,7 @@ int tp_mlp_create(tp_mlp** out, const double* params, void* cuda_stream) {
   tp_mlp* a = nullptr;
   TP_API_BEGIN
   a = new tp_mlp();
+  TP_CUDA_TRY(cudaGetDevice(&a->device));
   if (cuda_stream) {
     a->s = static_cast<cudaStream_t>(cuda_stream);
   } else {

@@ -6,6 +6,7 @@
 #include <cstring>
 #include <map>
 
+#include "in_place.cuh"
 #include "mlp_stage.cuh"
 #include "planes.cuh"
 
@@ -107,11 +108,45 @@ static void coupling_planes() {
   CHECK(g_device.empty());
 }
 
+// what a pointer query would say: one allocation of 4096 bytes at 1 << 40
+static CUmemorytype g_type;
+static int g_owner;
+static CUresult fake_query(unsigned n, CUpointer_attribute* what, void** to, CUdeviceptr) {
+  for (unsigned k = 0; k < n; ++k) {
+    if (what[k] == CU_POINTER_ATTRIBUTE_MEMORY_TYPE) *static_cast<CUmemorytype*>(to[k]) = g_type;
+    if (what[k] == CU_POINTER_ATTRIBUTE_RANGE_START_ADDR)
+      *static_cast<CUdeviceptr*>(to[k]) = CUdeviceptr(1) << 40;
+    if (what[k] == CU_POINTER_ATTRIBUTE_RANGE_SIZE) *static_cast<size_t*>(to[k]) = 4096;
+    if (what[k] == CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL) *static_cast<int*>(to[k]) = g_owner;
+  }
+  return CUDA_SUCCESS;
+}
+
+// a kernel takes only aligned memory of its own device, inside one allocation
+static void in_place() {
+  const char* base = reinterpret_cast<char*>(size_t(1) << 40);
+  auto usable = [&](int device, size_t byte, size_t n) {
+    return tp::usable_in_place(fake_query, device, reinterpret_cast<const double*>(base + byte), n);
+  };
+  g_type = CU_MEMORYTYPE_DEVICE;
+  g_owner = 1;
+  CHECK(usable(1, 0, 512) && usable(1, 8, 511) && usable(1, 4088, 1));
+  CHECK(!usable(0, 0, 512));                         // another GPU's
+  CHECK(!usable(1, 8, 512) && !usable(1, 0, 513));   // past the end
+  CHECK(!usable(1, 4, 1));                           // unaligned
+  g_owner = 0;
+  CHECK(usable(0, 0, 512) && !usable(1, 0, 512));
+  g_type = CU_MEMORYTYPE_HOST;
+  CHECK(!usable(0, 0, 1));
+  CHECK(!tp::usable_in_place<double>(nullptr, 0, nullptr, 1));
+}
+
 int main(int, char** argv) {
   const struct {
     const char* name;
     void (*run)();
-  } checks[] = {{"mlp_growth", mlp_growth}, {"coupling_planes", coupling_planes}};
+  } checks[] = {{"mlp_growth", mlp_growth}, {"coupling_planes", coupling_planes},
+                {"in_place", in_place}};
   for (const auto& c : checks)
     if (std::strcmp(argv[1], c.name) == 0) {
       c.run();
