@@ -559,7 +559,8 @@ double read_double(const double* d, double* host_pinned, cudaStream_t s) {
 }
 
 void ensure_workspace(tp_ctx* c, int restart) {
-  if (c->restart_alloc >= restart && c->Vb) return;
+  if (c->restart_alloc >= restart) return;
+  c->restart_alloc = 0;  // until every vector is there: a growth may run out of memory
   c->kpool.release();
   const long long n2 = 2ll * c->N;
   c->Vb = c->kpool.alloc<double>((size_t)(restart + 1) * n2);

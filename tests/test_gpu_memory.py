@@ -1,7 +1,7 @@
 """Calls on a device whose memory is nearly all taken give the results of the
 same calls with memory to spare: what is kept for speed alone is left out or
 given back."""
-import gc
+import ctypes as C
 
 import numpy as np
 import pytest
@@ -16,23 +16,27 @@ thermo = pytest.importorskip("paper_1902_00095_gb300.thermo")
 
 
 class Taken:
-    """Takes device memory until about `leave` bytes are free."""
+    """Takes device memory (in the process's context, past every pool) until at
+    most `leave` bytes and 2 MiB are free."""
 
     def __init__(self, leave):
         self.leave = leave
 
     def __enter__(self):
         torch.cuda.synchronize()
+        self.cuda = C.CDLL("libcuda.so.1")
         self.held = []
-        for block in (1 << 33, 1 << 28, 12 << 20):
+        for block in (1 << 33, 1 << 28, 1 << 21):
             while torch.cuda.mem_get_info()[0] >= self.leave + block:
-                self.held.append(torch.empty(block, dtype=torch.uint8, device="cuda"))
+                p = C.c_uint64()
+                if self.cuda.cuMemAlloc_v2(C.byref(p), C.c_size_t(block)) != 0:
+                    break
+                self.held.append(p)
         return self
 
     def __exit__(self, *exc):
-        self.held = None
-        gc.collect()
-        torch.cuda.empty_cache()
+        for p in self.held:
+            self.cuda.cuMemFree_v2(p)
 
 
 def solver(shape, seed=4):
@@ -57,5 +61,20 @@ def test_no_room_for_coupling_planes():
             assert np.array_equal(s.export_system()[4], scales)
     s.build(variant=1)
     y = s.solve(rtol=1e-8)
+    assert y[2]["iters"] == x[2]["iters"] and np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1])
+    s.close()
+
+
+# 3,840 cells: the Krylov vectors lie in pool chunks of 4 to 16 MiB, the larger
+# workspace's first vectors fit those that are there and its last ones do not
+def test_krylov_workspace_that_could_not_grow():
+    s = solver((16, 16, 15))
+    s.build()
+    x = s.solve(rtol=1e-8, restart=30)
+    with Taken(0):
+        with pytest.raises(thermo.ThermoError) as e:
+            s.solve(rtol=1e-8, restart=100)
+        assert e.value.status == thermo.TP_ENOMEM
+    y = s.solve(rtol=1e-8, restart=30)
     assert y[2]["iters"] == x[2]["iters"] and np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1])
     s.close()
