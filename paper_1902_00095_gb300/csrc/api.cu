@@ -1132,11 +1132,12 @@ void extract_blocks(tp_ctx* c) {
 // of the rows falling back switches the whole matrix back to plain S~
 void learned_features(tp_ctx* c) {
   cudaStream_t s = c->s;
-  if (!c->feat) {
-    c->feat = c->lpool.alloc<float>((size_t)c->N * kMlpIn);
+  if (!c->feat) {  // set last: an earlier one may run out of memory
+    c->lpool.release();
     c->mlp_out = c->lpool.alloc<float>((size_t)c->N * kMlpOut);
     c->S_learned = c->lpool.alloc<double>(c->nnzb);
     c->nbad = c->lpool.alloc<int>(1);
+    c->feat = c->lpool.alloc<float>((size_t)c->N * kMlpIn);
   }
   extract_blocks(c);
   launch_equation_scales(c->N, c->dpos, c->App, c->ATT, c->tmpN, c->partials, c->nparts,

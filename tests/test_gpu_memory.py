@@ -78,3 +78,19 @@ def test_krylov_workspace_that_could_not_grow():
     y = s.solve(rtol=1e-8, restart=30)
     assert y[2]["iters"] == x[2]["iters"] and np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1])
     s.close()
+
+
+# 800,000 cells: 26 MB for the network's outputs, 45 MB for S~, 77 MB of features
+def test_no_room_for_the_learned_work_arrays():
+    s = solver((100, 100, 80))
+    for leave in (85 << 20, 40 << 20):
+        with Taken(leave):
+            for _ in range(2):
+                with pytest.raises(thermo.ThermoError) as e:
+                    s.learned_features()
+                assert e.value.status == thermo.TP_ENOMEM
+    X = s.learned_features()
+    s.close()
+    r = solver((100, 100, 80))
+    assert np.array_equal(X, r.learned_features())
+    r.close()
