@@ -381,7 +381,11 @@ int  tp_learned_status(tp_ctx* ctx, int* fallback_rows, int* global_fallback);
  * A_Tp z)_i for the rows i of column j. Host outputs entry [ncols][7]
  * (pattern entry index of (i, j), -1 padding) and value [ncols][7];
  * iters = total FGMRES iterations. TP_NOT_CONVERGED if a solve stopped
- * above rtol. */
+ * above rtol. On grids of at most 131072 cells several columns are solved side
+ * by side; each of up to 8 solves in work keeps 61 vectors and a second set of
+ * level vectors with the context (some 90 MB at 131072 cells). Where memory
+ * does not reach for them there are fewer, or one solve after the other, and
+ * they are freed when another allocation of the context needs the memory. */
 int  tp_probe_schur_columns(tp_ctx* ctx, const int* cols, int ncols, double rtol,
                             int* entry, double* value, int* iters);
 

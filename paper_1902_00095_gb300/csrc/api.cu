@@ -968,10 +968,10 @@ int tp_probe_schur_columns(tp_ctx* c, const int* cols, int ncols, double rtol, i
   if (!c || !cols || ncols < 0 || !entry || !value || !(rtol > 0.0)) return TP_EINVAL;
   if (!c->built) return TP_ESTATE;
   TP_API_BEGIN
-  if (tp::column_lanes_usable(c, ncols)) {
-    int good = 0;  // columns before the first index out of range
-    while (good < ncols && cols[good] >= 0 && cols[good] < c->N) ++good;
-    const int st = tp::probe_schur_columns_lanes(c, cols, good, rtol, 500, entry, value,
+  int good = 0;  // columns before the first index out of range
+  while (good < ncols && cols[good] >= 0 && cols[good] < c->N) ++good;
+  if (const int lanes = tp::ready_column_lanes(c, good)) {
+    const int st = tp::probe_schur_columns_lanes(c, lanes, cols, good, rtol, 500, entry, value,
                                                  good < ncols ? nullptr : iters);
     return good < ncols ? TP_EINVAL : st;
   }
@@ -1132,13 +1132,14 @@ void extract_blocks(tp_ctx* c) {
 // of the rows falling back switches the whole matrix back to plain S~
 void learned_features(tp_ctx* c) {
   cudaStream_t s = c->s;
-  if (!c->feat) {  // set last: an earlier one may run out of memory
-    c->lpool.release();
-    c->mlp_out = c->lpool.alloc<float>((size_t)c->N * kMlpOut);
-    c->S_learned = c->lpool.alloc<double>(c->nnzb);
-    c->nbad = c->lpool.alloc<int>(1);
-    c->feat = c->lpool.alloc<float>((size_t)c->N * kMlpIn);
-  }
+  if (!c->feat)
+    with_memory_given_back(c, [&] {  // feat last: an earlier one may run out of memory
+      c->lpool.release();
+      c->mlp_out = c->lpool.alloc<float>((size_t)c->N * kMlpOut);
+      c->S_learned = c->lpool.alloc<double>(c->nnzb);
+      c->nbad = c->lpool.alloc<int>(1);
+      c->feat = c->lpool.alloc<float>((size_t)c->N * kMlpIn);
+    });
   extract_blocks(c);
   launch_equation_scales(c->N, c->dpos, c->App, c->ATT, c->tmpN, c->partials, c->nparts,
                          c->scales, s);
@@ -1256,8 +1257,7 @@ static void on_both(tp_ctx* c, FP on_pp, FS on_S) {
   TP_CUDA_TRY(cudaStreamWaitEvent(s, c->ev_join, 0));
 }
 
-void build_device(tp_ctx* c, const tp_precond_opts& o) {
-  cudaStream_t s = c->s;
+static void drop_graph(tp_ctx* c) {
   if (c->pc_graph) {
     cudaGraphExecDestroy(c->pc_graph);
     c->pc_graph = nullptr;
@@ -1266,15 +1266,76 @@ void build_device(tp_ctx* c, const tp_precond_opts& o) {
     cudaGraphDestroy(c->pc_graph_tmpl);
     c->pc_graph_tmpl = nullptr;
   }
+  c->probe_nodes.clear();
+  c->probe_set = 0;
+}
+
+// the block preconditioner of the last build as a graph
+static void record_graph(tp_ctx* c) {
+  cudaStream_t s = c->s;
+  cudaGraph_t graph = nullptr;
+  TP_CUDA_TRY(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+  g_capturing = true;
+  try {
+    precond_record(c, s);
+  } catch (...) {
+    g_capturing = false;
+    cudaStreamEndCapture(s, &graph);
+    if (graph) cudaGraphDestroy(graph);
+    throw;
+  }
+  g_capturing = false;
+  TP_CUDA_TRY(cudaStreamEndCapture(s, &graph));
+  size_t nodes = 0;
+  TP_CUDA_TRY(cudaGraphGetNodes(graph, nullptr, &nodes));
+  std::vector<cudaGraphNode_t> list(nodes);
+  if (nodes) TP_CUDA_TRY(cudaGraphGetNodes(graph, list.data(), &nodes));
+  long long kernels = 0;
+  for (cudaGraphNode_t nd : list) {
+    cudaGraphNodeType ty;
+    TP_CUDA_TRY(cudaGraphNodeGetType(nd, &ty));
+    if (ty == cudaGraphNodeTypeKernel) ++kernels;
+    if (ty == cudaGraphNodeTypeEventRecord) {
+      cudaEvent_t ev = nullptr;
+      TP_CUDA_TRY(cudaGraphEventRecordNodeGetEvent(nd, &ev));
+      for (int k = 0; k < 2 * tp::Probe::kMaxPairs; ++k)
+        if (c->probe.created && c->probe.ev[0][k] == ev) c->probe_nodes.push_back({nd, k});
+    }
+  }
+  c->pc_graph_kernels = kernels;
+  cudaError_t e = cudaGraphInstantiate(&c->pc_graph, graph, 0);
+  if (e != cudaSuccess) {
+    cudaGraphDestroy(graph);
+    c->pc_graph = nullptr;
+    c->probe_nodes.clear();
+    fail(TP_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+  }
+  c->pc_graph_tmpl = graph;
+}
+
+bool give_back(tp_ctx* c) {
+  if (!c->lanes.empty()) {
+    drop_column_lanes(c);
+    return true;
+  }
+  if (!c->planes.ApT) return false;
+  TP_CUDA_TRY(cudaStreamSynchronize(c->s));
+  const bool recorded = c->pc_graph != nullptr;  // it reads the planes
+  drop_graph(c);
+  c->planes.give_back();
+  if (recorded) record_graph(c);
+  return true;
+}
+
+static void build_once(tp_ctx* c, const tp_precond_opts& o) {
+  cudaStream_t s = c->s;
+  drop_graph(c);
   if (c->vc_graph) {
     cudaGraphExecDestroy(c->vc_graph);
     c->vc_graph = nullptr;
   }
   stale_column_lanes(c);
-  c->probe_nodes.clear();
-  c->probe_set = 0;
   c->built = false;
-  c->planes.refused = false;
   extract_blocks(c);
   launch_equation_scales(c->N, c->dpos, c->App, c->ATT, c->tmpN, c->partials, c->nparts,
                          c->scales, s);
@@ -1323,48 +1384,14 @@ void build_device(tp_ctx* c, const tp_precond_opts& o) {
   c->hpp->probe_level = c->probe_which == 3 ? 1 : 0;
   c->hS->probe = c->probe_which == 1 ? &c->probe : nullptr;
   c->hS->probe_level = 0;
-  if (o.use_graphs) {
-    cudaGraph_t graph = nullptr;
-    TP_CUDA_TRY(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-    g_capturing = true;
-    try {
-      precond_record(c, s);
-    } catch (...) {
-      g_capturing = false;
-      cudaStreamEndCapture(s, &graph);
-      if (graph) cudaGraphDestroy(graph);
-      throw;
-    }
-    g_capturing = false;
-    TP_CUDA_TRY(cudaStreamEndCapture(s, &graph));
-    size_t nodes = 0;
-    TP_CUDA_TRY(cudaGraphGetNodes(graph, nullptr, &nodes));
-    std::vector<cudaGraphNode_t> list(nodes);
-    if (nodes) TP_CUDA_TRY(cudaGraphGetNodes(graph, list.data(), &nodes));
-    long long kernels = 0;
-    for (cudaGraphNode_t nd : list) {
-      cudaGraphNodeType ty;
-      TP_CUDA_TRY(cudaGraphNodeGetType(nd, &ty));
-      if (ty == cudaGraphNodeTypeKernel) ++kernels;
-      if (ty == cudaGraphNodeTypeEventRecord) {
-        cudaEvent_t ev = nullptr;
-        TP_CUDA_TRY(cudaGraphEventRecordNodeGetEvent(nd, &ev));
-        for (int k = 0; k < 2 * tp::Probe::kMaxPairs; ++k)
-          if (c->probe.created && c->probe.ev[0][k] == ev) c->probe_nodes.push_back({nd, k});
-      }
-    }
-    c->pc_graph_kernels = kernels;
-    cudaError_t e = cudaGraphInstantiate(&c->pc_graph, graph, 0);
-    if (e != cudaSuccess) {
-      cudaGraphDestroy(graph);
-      c->pc_graph = nullptr;
-      c->probe_nodes.clear();
-      fail(TP_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-    }
-    c->pc_graph_tmpl = graph;
-  }
+  if (o.use_graphs) record_graph(c);
   TP_CUDA_TRY(cudaStreamSynchronize(s));
   c->built = true;
+}
+
+void build_device(tp_ctx* c, const tp_precond_opts& o) {
+  c->planes.refused = false;
+  with_memory_given_back(c, [&] { build_once(c, o); });
 }
 
 void refresh_device(tp_ctx* c) {

@@ -558,8 +558,7 @@ double read_double(const double* d, double* host_pinned, cudaStream_t s) {
   return *host_pinned;
 }
 
-void ensure_workspace(tp_ctx* c, int restart) {
-  if (c->restart_alloc >= restart) return;
+void lay_out_workspace(tp_ctx* c, int restart) {
   c->restart_alloc = 0;  // until every vector is there: a growth may run out of memory
   c->kpool.release();
   const long long n2 = 2ll * c->N;
@@ -582,6 +581,11 @@ void ensure_workspace(tp_ctx* c, int restart) {
   c->oparts = c->kpool.alloc<double>((size_t)orth_grid(c, 2ll * c->N) + 16);
   c->reorth = c->kpool.alloc<int>(4);
   c->restart_alloc = restart;
+}
+
+void ensure_workspace(tp_ctx* c, int restart) {
+  if (c->restart_alloc < restart)
+    with_memory_given_back(c, [&] { lay_out_workspace(c, restart); });
 }
 
 // y = A x (scalar CSR, one thread per row); z = x
@@ -1040,27 +1044,39 @@ bool lane_advance(tp_ctx* c, ColumnLane& t, double rtol, int maxit) {
 
 }  // namespace
 
-bool column_lanes_usable(const tp_ctx* c, int ncols) {
-  return ncols > 1 && c->N <= kColumnLaneRows && c->opts.use_graphs && !c->hpp->probe &&
-         c->hpp->tail_first < 0;
+// Lanes for ncols columns, prepared for the last build. A lane that cannot be
+// had (memory, as a rule: 61 vectors and a second set of level vectors, 90 MB at
+// 131072 cells) leaves the columns to those before it, and those after it are
+// given up; fewer than two are no better than one solve after the other, which
+// needs the context's own workspace only.
+int ready_column_lanes(tp_ctx* c, int ncols) {
+  if (ncols < 2 || c->N > kColumnLaneRows || !c->opts.use_graphs || c->hpp->probe ||
+      c->hpp->tail_first >= 0)
+    return 0;
+  const int want = ncols < kColumnLanes ? ncols : kColumnLanes;
+  int l = 0;
+  try {
+    if (!c->ev_lanes)
+      TP_CUDA_TRY(cudaEventCreateWithFlags(&c->ev_lanes, cudaEventDisableTiming));
+    for (; l < want; ++l) {
+      if (l == (int)c->lanes.size()) {
+        c->lanes.emplace_back(new ColumnLane());
+        open_lane(*c->lanes.back());
+      }
+      if (c->lanes[l]->stale) prepare_lane(c, *c->lanes[l]);
+    }
+  } catch (const Error&) {
+    cudaGetLastError();
+    if (l < 2) l = 0;
+    c->lanes.resize(l);
+  }
+  return l;
 }
 
-int probe_schur_columns_lanes(tp_ctx* c, const int* cols, int ncols, double rtol, int maxit,
-                              int* entry, double* value, int* iters) {
-  const int nl = ncols < kColumnLanes ? ncols : kColumnLanes;
-  if (!c->ev_lanes)
-    TP_CUDA_TRY(cudaEventCreateWithFlags(&c->ev_lanes, cudaEventDisableTiming));
-  while ((int)c->lanes.size() < nl) {
-    c->lanes.emplace_back(new ColumnLane());
-    try {
-      open_lane(*c->lanes.back());
-    } catch (...) {
-      c->lanes.pop_back();
-      throw;
-    }
-  }
-  for (int l = 0; l < nl; ++l)
-    if (c->lanes[l]->stale) prepare_lane(c, *c->lanes[l]);
+void drop_column_lanes(tp_ctx* c) { c->lanes.clear(); }
+
+int probe_schur_columns_lanes(tp_ctx* c, int nl, const int* cols, int ncols, double rtol,
+                              int maxit, int* entry, double* value, int* iters) {
   TP_CUDA_TRY(cudaEventRecord(c->ev_lanes, c->s));
   int next = 0, busy = 0, total = 0, status = TP_OK;
   auto take = [&](ColumnLane& t) {

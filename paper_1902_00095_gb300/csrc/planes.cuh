@@ -28,6 +28,12 @@ struct CouplingPlanes {
     }
     return true;
   }
+  // for an allocation that cannot be done without; nothing may be reading them
+  void give_back() {
+    ApT = ATp = nullptr;
+    refused = true;
+    pool.free_all();
+  }
 };
 
 }  // namespace tp

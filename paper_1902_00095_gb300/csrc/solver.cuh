@@ -125,11 +125,30 @@ int newton_step(tp_ctx* c, double dt, const tp_precond_opts& popts, const tp_new
 int scalar_fgmres(tp_ctx* c, Hierarchy& h, const DevCSR& A, const double* b, double* x,
                   double rtol, int maxit, int restart);
 int probe_schur_column(tp_ctx* c, int j, double rtol, int maxit, int* entry, double* value);
-// the same for several columns side by side: host outputs, total iterations;
-// TP_OK or TP_NOT_CONVERGED
-bool column_lanes_usable(const tp_ctx* c, int ncols);
-int probe_schur_columns_lanes(tp_ctx* c, const int* cols, int ncols, double rtol, int maxit,
-                              int* entry, double* value, int* iters);
+// the same for several columns side by side on `nl` lanes (ready_column_lanes:
+// 0 where they cannot be used or memory for fewer than two is left): host
+// outputs, total iterations; TP_OK or TP_NOT_CONVERGED
+int ready_column_lanes(tp_ctx* c, int ncols);
+int probe_schur_columns_lanes(tp_ctx* c, int nl, const int* cols, int ncols, double rtol,
+                              int maxit, int* entry, double* value, int* iters);
 void stale_column_lanes(tp_ctx* c);
+void drop_column_lanes(tp_ctx* c);
+// Frees memory that the context keeps for speed alone: the lanes, then the
+// coupling planes (the recorded preconditioner is recorded anew without them).
+// False when there is none.
+bool give_back(tp_ctx* c);
+// f, again after each give_back() while it runs out of device memory: what is
+// kept for speed makes no call fail that would do without it
+template <class F>
+void with_memory_given_back(tp_ctx* c, F f) {
+  while (true) {
+    try {
+      f();
+      return;
+    } catch (const Error& e) {
+      if (e.code != TP_ENOMEM || !give_back(c)) throw;
+    }
+  }
+}
 void learned_features(tp_ctx* c);  // features of the last assembly into c->feat
 }  // namespace tp

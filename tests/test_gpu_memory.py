@@ -39,6 +39,11 @@ class Taken:
             self.cuda.cuMemFree_v2(p)
 
 
+def free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
 def solver(shape, seed=4):
     prob = make_problem("tiny", shape=shape, seed=seed)
     p, T = perturbed_state(prob, seed=seed + 1)
@@ -94,3 +99,67 @@ def test_no_room_for_the_learned_work_arrays():
     r = solver((100, 100, 80))
     assert np.array_equal(X, r.learned_features())
     r.close()
+
+
+# 131,072 cells: some 90 MB a lane. Room for a few lanes, for none, and again
+# for all on the same context
+def test_columns_with_room_for_few_lanes():
+    s = solver((64, 64, 32))
+    s.build()
+    s.solve(rtol=1e-8)  # the context's own workspace
+    cols = np.arange(0, s.N, 13001, dtype=np.int32)
+    assert cols.size > 8
+    one = [s.probe_schur_columns([c], rtol=1e-10) for c in cols]
+    for leave in (16 << 20, 130 << 20, 300 << 20):
+        with Taken(leave):
+            entry, value, its, st = s.probe_schur_columns(cols, rtol=1e-10)
+        assert st == 0 and its == sum(o[2] for o in one)
+        assert np.array_equal(entry, np.concatenate([o[0] for o in one]))
+        assert np.array_equal(value, np.concatenate([o[1] for o in one]))
+    s.close()
+
+
+# a larger Krylov workspace in 40 MB less than it takes: it fits only into what the
+# lanes (131,072 cells), or the coupling planes (90 MB at 800,000 cells, with the
+# graph recorded anew), give back
+@pytest.mark.parametrize("shape", [(64, 64, 32), (100, 100, 80)])
+def test_memory_kept_for_speed_is_given_back(shape):
+    r = solver(shape)
+    r.build()
+    r.solve(rtol=1e-8, restart=30)
+    f = free()
+    x = r.solve(rtol=1e-8, restart=31)
+    taken = f - free()
+    r.close()
+    s = solver(shape)
+    s.build()
+    s.solve(rtol=1e-8, restart=30)
+    cols = [0, 1, 2]
+    c0 = s.probe_schur_columns(cols, rtol=1e-10)
+    with Taken(taken - (40 << 20)):
+        y = s.solve(rtol=1e-8, restart=31)
+    z = s.solve(rtol=1e-8, restart=31)
+    c1 = s.probe_schur_columns(cols, rtol=1e-10)
+    s.build()
+    w = s.solve(rtol=1e-8, restart=31)
+    s.close()
+    assert np.array_equal(c0[0], c1[0]) and np.array_equal(c0[1], c1[1])
+    for a in (y, z, w):
+        assert a[2]["iters"] == x[2]["iters"]
+        assert np.array_equal(a[0], x[0]) and np.array_equal(a[1], x[1])
+
+
+# 800,000 cells, 90 MB of planes: a first build in 40 MB less than it takes
+def test_build_in_the_memory_of_one_without_planes():
+    r = solver((100, 100, 80))
+    f = free()
+    r.build()
+    taken = f - free()
+    x = r.solve(rtol=1e-8)
+    r.close()
+    s = solver((100, 100, 80))
+    with Taken(taken - (40 << 20)):
+        s.build()
+    y = s.solve(rtol=1e-8)
+    s.close()
+    assert y[2]["iters"] == x[2]["iters"] and np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1])
