@@ -4,7 +4,7 @@
 #include <cmath>
 #include <cstring>
 #include <algorithm>
-#include <thread>
+#include "fork_join.cuh"
 #include "in_place.cuh"
 #include "mlp_stage.cuh"
 #include "solver.cuh"
@@ -1219,8 +1219,7 @@ void schur_diag_values(tp_ctx* c, bool symbolic) {
 // thread on a second stream while this thread does A_pp's (setups and
 // refreshes are chains of small kernels with host round trips, so they
 // overlap; the four refreshes of a 64x64x32 Newton step one after the other
-// cost it 57 instead of 54 ms). Both see everything enqueued on the context stream before
-// the call, and it waits for both.
+// cost it 57 instead of 54 ms).
 template <class FP, class FS>
 static void on_both(tp_ctx* c, FP on_pp, FS on_S) {
   cudaStream_t s = c->s;
@@ -1229,32 +1228,7 @@ static void on_both(tp_ctx* c, FP on_pp, FS on_S) {
     TP_CUDA_TRY(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
     TP_CUDA_TRY(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
   }
-  TP_CUDA_TRY(cudaEventRecord(c->ev_fork, s));
-  TP_CUDA_TRY(cudaStreamWaitEvent(c->s2, c->ev_fork, 0));
-  Error terr{TP_OK, ""};
-  bool tfail = false;
-  std::thread th([&]() {
-    try {
-      TP_CUDA_TRY(cudaSetDevice(c->device));
-      on_S(c->s2);
-    } catch (const Error& e) {
-      terr = e;
-      tfail = true;
-    } catch (...) {
-      terr = Error{TP_ECUDA, "Schur hierarchy setup failed"};
-      tfail = true;
-    }
-  });
-  try {
-    on_pp(s);
-  } catch (...) {
-    th.join();
-    throw;
-  }
-  th.join();
-  if (tfail) throw terr;
-  TP_CUDA_TRY(cudaEventRecord(c->ev_join, c->s2));
-  TP_CUDA_TRY(cudaStreamWaitEvent(s, c->ev_join, 0));
+  fork_join(c->device, s, c->s2, c->ev_fork, c->ev_join, on_pp, on_S);
 }
 
 static void drop_graph(tp_ctx* c) {

@@ -6,6 +6,7 @@
 #include <cstring>
 #include <map>
 
+#include "fork_join.cuh"
 #include "in_place.cuh"
 #include "mlp_stage.cuh"
 #include "planes.cuh"
@@ -39,6 +40,16 @@ cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return cudaMallocHost(
 cudaError_t cudaFreeHost(void* p) {
   g_pinned.erase(static_cast<char*>(p));
   std::free(p);
+  return cudaSuccess;
+}
+static const char* g_where[8];  // what s and s2 were made to wait for, in order
+static int g_waits = 0;
+cudaError_t cudaSetDevice(int) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
+  g_where[g_waits++ & 7] = reinterpret_cast<size_t>(s) == 1
+                               ? (reinterpret_cast<size_t>(e) == 4 ? "s:join" : "s:fork")
+                               : (reinterpret_cast<size_t>(e) == 3 ? "s2:fork" : "s2:join");
   return cudaSuccess;
 }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
@@ -141,12 +152,44 @@ static void in_place() {
   CHECK(!tp::usable_in_place<double>(nullptr, 0, nullptr, 1));
 }
 
+// the first stream waits for the second's work however the two sides end, and
+// an exception of either leaves the call after both are done
+static void fork_join() {
+  const auto s = reinterpret_cast<cudaStream_t>(1), s2 = reinterpret_cast<cudaStream_t>(2);
+  const auto fork = reinterpret_cast<cudaEvent_t>(3), join = reinterpret_cast<cudaEvent_t>(4);
+  for (int fail = 0; fail < 4; ++fail) {
+    g_waits = 0;
+    int done = 0, code = 0, waits_on_s = -1, waits_on_s2 = -1;
+    try {
+      tp::fork_join(
+          0, s, s2, fork, join,
+          [&](cudaStream_t t) {
+            CHECK(t == s);
+            waits_on_s = g_waits;
+            if (fail & 1) tp::fail(TP_ENOMEM, "first");
+          },
+          [&](cudaStream_t t) {
+            CHECK(t == s2);
+            waits_on_s2 = g_waits;
+            done = 1;
+            if (fail & 2) tp::fail(TP_SETUP_FAILED, "second");
+          });
+    } catch (const tp::Error& e) {
+      code = e.code;
+    }
+    CHECK(done && waits_on_s == 1 && waits_on_s2 == 1);  // s2 waits for s before either
+    CHECK(code == (fail & 1 ? TP_ENOMEM : fail & 2 ? TP_SETUP_FAILED : 0));
+    CHECK(g_waits == 2 && !std::strcmp(g_where[0], "s2:fork") && !std::strcmp(g_where[1], "s:join"));
+  }
+}
+
 int main(int, char** argv) {
   const struct {
     const char* name;
     void (*run)();
   } checks[] = {{"mlp_growth", mlp_growth}, {"coupling_planes", coupling_planes},
-                {"in_place", in_place}};
+                {"in_place", in_place},
+                {"fork_join", fork_join}};
   for (const auto& c : checks)
     if (std::strcmp(argv[1], c.name) == 0) {
       c.run();

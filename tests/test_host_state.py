@@ -1,6 +1,7 @@
 """Host logic of the CUDA library's headers (buffers after a failed allocation,
-use of a caller's arrays), compiled with the host compiler against a fake CUDA
-runtime: no GPU, and no fault on one, is needed to see it."""
+use of a caller's arrays, joining of two streams), compiled with the host
+compiler against a fake CUDA runtime: no GPU, and no fault on one, is needed to
+see it."""
 import os
 import shutil
 import subprocess
@@ -27,7 +28,7 @@ def checks(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("name", ["mlp_growth", "coupling_planes", "in_place"])
+@pytest.mark.parametrize("name", ["mlp_growth", "coupling_planes", "in_place", "fork_join"])
 def test_host_state(checks, name):
     r = subprocess.run([checks, name], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
