@@ -27,6 +27,7 @@
 // low occupancy (shared memory and registers leave 19-28 of 64 warps per SM;
 // the 8-lane form also keeps the FP64 pipe half busy, mostly divisions).
 #include "amg_dev.cuh"
+#include "per_device.cuh"
 
 namespace tp {
 
@@ -510,12 +511,8 @@ void launch_tier(int blocks_per_sm, int sms, int n, const int* list, const int* 
                  double* tval, int* olist, int* ocnt, cudaStream_t s) {
   auto kern = k_interp<EXT, G, R, SET, ENT, KM, RL, WARPS>;
   constexpr size_t smem = WARPS * sizeof(InterpRows<R, SET, ENT, KM, RL>);
-  static const bool attr = [&]() {
-    TP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
-    return true;
-  }();
-  (void)attr;
+  static PerDevice<bool> allowed;
+  allow_smem(allowed, kern, smem);
   long long blocks = ((long long)n + R * WARPS - 1) / (R * WARPS);
   if (list && blocks > (long long)blocks_per_sm * sms) blocks = (long long)blocks_per_sm * sms;
   kern<<<(int)blocks, 32 * WARPS, smem, s>>>(n, list, nlist, A.rowptr, A.col, A.val, dpos,

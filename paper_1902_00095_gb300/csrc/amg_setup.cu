@@ -8,6 +8,7 @@
 // its distance-two extended+i form; all structure-deciding arithmetic uses
 // __dmul_rn / __dadd_rn / __ddiv_rn in a fixed ascending-column order.
 #include "amg_dev.cuh"
+#include "per_device.cuh"
 #include <cmath>
 #include <algorithm>
 
@@ -15,7 +16,6 @@ namespace tp {
 
 namespace {
 
-int setup_sms();
 long long resident_threads();
 
 // (d > 0 && a < 0) || (d < 0 && a > 0), decided on the bit patterns: both
@@ -1266,27 +1266,15 @@ int pick_lanes(const DevCSR& A) {
   return l > 16 ? 16 : l;
 }
 
-// threads resident on the whole device at full occupancy, once per process
+// threads resident on the whole device at full occupancy
 long long resident_threads() {
-  static const long long r = []() {
-    int dev = 0, sms = 0, thr = 0;
+  static PerDevice<long long> threads;
+  return threads([] {
+    int dev = 0, thr = 0;
     TP_CUDA_TRY(cudaGetDevice(&dev));
-    TP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     TP_CUDA_TRY(cudaDeviceGetAttribute(&thr, cudaDevAttrMaxThreadsPerMultiProcessor, dev));
-    return (long long)sms * thr;
-  }();
-  return r;
-}
-
-// SM count of the current device, once per process (thread-safe)
-int setup_sms() {
-  static const int sms = []() {
-    int dev = 0, v = 0;
-    TP_CUDA_TRY(cudaGetDevice(&dev));
-    TP_CUDA_TRY(cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev));
-    return v;
-  }();
-  return sms;
+    return (long long)device_sms() * thr;
+  });
 }
 
 int read_int(const int* d, cudaStream_t s) {
@@ -1431,7 +1419,7 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
     // rows per block of 256 threads: all 256 where that leaves eight blocks per
     // SM, fewer on small levels (at least one per lane group)
     const int rows_min = wrow ? 8 : 32;
-    const int rows = std::max(rows_min, std::min(256, n / (8 * setup_sms())));
+    const int rows = std::max(rows_min, std::min(256, n / (8 * device_sms())));
     const int gr = grid_for(n, rows);
     int rounds = 0;
     while (true) {
@@ -1469,7 +1457,7 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
     // by kernels of their own
     DevCSR P;
     const bool one_pass =
-        opts.pmax > 0 && truncated_interpolation(A, opts.interp != 0, setup_sms(), cur.dpos,
+        opts.pmax > 0 && truncated_interpolation(A, opts.interp != 0, device_sms(), cur.dpos,
                                                  cur.strong, cur.cf, cidx, nc, opts.pmax, pool,
                                                  scratch, P, s);
     int* cnt = nullptr;
@@ -1493,7 +1481,7 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
       TP_LAUNCH_CHECK();
       {
         long long blocks = ((long long)n + kClsWarps - 1) / kClsWarps;
-        if (blocks > 8LL * setup_sms()) blocks = 8LL * setup_sms();
+        if (blocks > 8LL * device_sms()) blocks = 8LL * device_sms();
         k_classical_fill_warp<<<(int)blocks, 32 * kClsWarps, 0, s>>>(
             n, A.rowptr, A.col, A.val, cur.dpos, cur.strong, cur.cf, cidx, P.rowptr, P.col,
             P.val);
@@ -1511,7 +1499,7 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
       TP_LAUNCH_CHECK();
       {
         long long blocks = ((long long)n + kSetWarps - 1) / kSetWarps;
-        if (blocks > 8LL * setup_sms()) blocks = 8LL * setup_sms();
+        if (blocks > 8LL * device_sms()) blocks = 8LL * device_sms();
         k_extpi_sets_warp<<<(int)blocks, 32 * kSetWarps, 0, s>>>(n, A.rowptr, A.col, cur.strong,
                                                                  cur.cf, off, ub, buf, cnt);
         TP_LAUNCH_CHECK();

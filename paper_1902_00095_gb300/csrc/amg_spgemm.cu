@@ -7,6 +7,7 @@
 // kernel takes the row.
 #include <algorithm>
 #include "amg_dev.cuh"
+#include "per_device.cuh"
 
 namespace tp {
 
@@ -282,12 +283,8 @@ void launch_group(const DevCSR& A, const DevCSR& B, const int* list, const int* 
   constexpr int WARPS = 4, NG = 32 / G;
   constexpr size_t smem = WARPS * sizeof(GroupRows<G, CAP, MAXU>);
   auto kern = k_spgemm_group<G, CAP, MAXU, WARPS, KNOWN>;
-  static const bool attr = [&]() {
-    TP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
-    return true;
-  }();
-  (void)attr;
+  static PerDevice<bool> allowed;
+  allow_smem(allowed, kern, smem);
   long long blocks = ((long long)A.n + WARPS * NG - 1) / (WARPS * NG);
   if (list && blocks > 16ll * sms) blocks = 16ll * sms;
   if (blocks < 1) blocks = 1;
@@ -672,18 +669,6 @@ __global__ void k_spgemm_compact(int n, const int* __restrict__ off,
 }
 
 
-// SM count of the current device, once per process (thread-safe; hierarchies
-// are set up concurrently)
-int spgemm_sms() {
-  static const int sms = []() {
-    int dev = 0, v = 0;
-    TP_CUDA_TRY(cudaGetDevice(&dev));
-    TP_CUDA_TRY(cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev));
-    return v;
-  }();
-  return sms;
-}
-
 }  // namespace
 
 // C = A B with the canonical summation order; C arrays allocated from `pool`.
@@ -704,20 +689,16 @@ DevCSR csr_product(const DevCSR& A, const DevCSR& B, Pool& pool, Pool& scratch, 
   int* cnt = scratch.alloc<int>(n + 1);
   const bool dense = B.m <= kDenseCap;
   if (dense) {
-    static const bool dense_attr = []() {
-      TP_CUDA_TRY(cudaFuncSetAttribute(k_spgemm_dense, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kDenseSmem));
-      return true;
-    }();
-    (void)dense_attr;
+    static PerDevice<bool> allowed;
+    allow_smem(allowed, k_spgemm_dense, kDenseSmem);
     long long blocks = ((long long)n + kDenseWarps - 1) / kDenseWarps;
-    if (blocks > 8LL * spgemm_sms()) blocks = 8LL * spgemm_sms();
+    if (blocks > 8LL * device_sms()) blocks = 8LL * device_sms();
     const size_t smem = (size_t)kDenseWarps * B.m * (sizeof(double) + 1);
     k_spgemm_dense<<<(int)blocks, 32 * kDenseWarps, smem, s>>>(
         n, B.m, A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, off, ccol, cval, cnt);
     TP_LAUNCH_CHECK();
   } else {
-    const int sms = spgemm_sms();
+    const int sms = device_sms();
     group_class<false>(false, A, B, (const int*)nullptr, (const int*)nullptr, kSpFirst,
                        (const int*)off, (const int*)ub, ccol, cval, cnt, list, counts,
                        (int*)nullptr, (int*)nullptr, sms, s);
@@ -730,12 +711,8 @@ DevCSR csr_product(const DevCSR& A, const DevCSR& B, Pool& pool, Pool& scratch, 
         A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, off, ub, olist, counts + 1, ccol, cval,
         cnt);
     TP_LAUNCH_CHECK();
-    static const bool big_attr = []() {
-      TP_CUDA_TRY(cudaFuncSetAttribute(
-          k_spgemm_rows_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpBigSmem));
-      return true;
-    }();
-    (void)big_attr;
+    static PerDevice<bool> allowed;
+    allow_smem(allowed, k_spgemm_rows_big, kSpBigSmem);
     k_spgemm_rows_big<<<n < sms ? n : sms, kSpBigThreads, kSpBigSmem, s>>>(
         n, A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, off, ub, blist, counts + 2, ccol, cval,
         cnt);
@@ -778,7 +755,7 @@ void csr_product_numeric(const DevCSR& A, const DevCSR& B, const DevCSR& C, Pool
   int* olist = scratch.alloc<int>(n + 1);
   int* counts = scratch.alloc<int>(3);
   TP_CUDA_TRY(cudaMemsetAsync(counts, 0, 3 * sizeof(int), s));
-  const int sms = spgemm_sms();
+  const int sms = device_sms();
   const int* rows = nullptr;
   const int* nrows = nullptr;
   if (C.nnz <= 48ll * n) {

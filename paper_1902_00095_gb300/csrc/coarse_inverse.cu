@@ -39,6 +39,7 @@
 #include <climits>
 
 #include "amg.cuh"
+#include "per_device.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -281,7 +282,8 @@ GjConfig probe_gj() {
 }  // namespace
 
 bool coarse_inverse_cluster(int n, const double* A, double* inv, int* err, cudaStream_t s) {
-  static const GjConfig g = probe_gj();
+  static PerDevice<GjConfig> config;
+  const GjConfig g = config(probe_gj);
   if (g.cluster == 0 || n < 1) return false;
   const int R = (n + g.cluster - 1) / g.cluster;
   const GjLayout lay(n, R);

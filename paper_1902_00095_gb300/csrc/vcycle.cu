@@ -17,6 +17,7 @@
 #include <type_traits>
 
 #include "amg.cuh"
+#include "per_device.cuh"
 
 namespace tp {
 
@@ -985,12 +986,8 @@ template <int W, class TV, class TB, class TO>
 void line_block(const Smooth& sm, const Level& v, const TB* b, const TV* xin, TO* xout,
                 cudaStream_t s) {
   auto kern = k_line_block<W, TV, TB, TO>;
-  static const bool attr = [&]() {
-    TP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kLineSmemMax));
-    return true;
-  }();
-  (void)attr;
+  static PerDevice<bool> allowed;
+  allow_smem(allowed, kern, kLineSmemMax);
   launch_pdl_smem(kern, (sm.line_nxy + W - 1) / W, kLineThreads,
                   line_block_smem<TV>(sm.line_nz, W), s, sm.line_nxy, sm.line_nz, v.A.n, v.ell_w,
                   v.ell_col, v.ell_nx, v.ell_nxy, Vals<TV>::E(v), v.A.rowptr, v.A.col,

@@ -26,6 +26,7 @@
 // read-only. Every thread of every CTA executes the same sequence of
 // barriers: loop bounds depend only on level sizes.
 #include "amg.cuh"
+#include "per_device.cuh"
 
 namespace tp {
 
@@ -268,8 +269,8 @@ int probe_cluster_size() {
 }  // namespace
 
 int tail_cluster_size() {
-  static const int c = probe_cluster_size();
-  return c;
+  static PerDevice<int> size;
+  return size(probe_cluster_size);
 }
 
 template <class TV>

@@ -9,6 +9,7 @@
 #include "fork_join.cuh"
 #include "in_place.cuh"
 #include "mlp_stage.cuh"
+#include "per_device.cuh"
 #include "planes.cuh"
 
 // ---------------------------------------------------------------- fake runtime
@@ -40,6 +41,20 @@ cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return cudaMallocHost(
 cudaError_t cudaFreeHost(void* p) {
   g_pinned.erase(static_cast<char*>(p));
   std::free(p);
+  return cudaSuccess;
+}
+static int g_dev = 0, g_attributes = 0;
+cudaError_t cudaGetDevice(int* d) {
+  *d = g_dev;
+  return cudaSuccess;
+}
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int d) {
+  *v = 100 + d;
+  return cudaSuccess;
+}
+cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int bytes) {
+  if (bytes < 0) return cudaErrorInvalidValue;
+  ++g_attributes;
   return cudaSuccess;
 }
 static const char* g_where[8];  // what s and s2 were made to wait for, in order
@@ -183,13 +198,37 @@ static void fork_join() {
   }
 }
 
+// a kernel's shared memory is allowed once on every device it is launched on,
+// and what a device answers is that device's
+static void per_device() {
+  static tp::PerDevice<bool> allowed;
+  const void* kernel = &g_dev;
+  for (int round = 0; round < 3; ++round)
+    for (g_dev = 0; g_dev < 4; ++g_dev) {
+      tp::allow_smem(allowed, kernel, 100 << 10);
+      CHECK(g_attributes == (round ? 4 : g_dev + 1));
+      CHECK(tp::device_sms() == 100 + g_dev);
+    }
+  static tp::PerDevice<bool> failing;
+  g_dev = 1;
+  bool threw = false;
+  try {
+    tp::allow_smem(failing, kernel, size_t(-1));
+  } catch (const tp::Error&) {
+    threw = true;
+  }
+  tp::allow_smem(failing, kernel, 1 << 10);  // tried again
+  CHECK(threw && g_attributes == 5);
+}
+
 int main(int, char** argv) {
   const struct {
     const char* name;
     void (*run)();
   } checks[] = {{"mlp_growth", mlp_growth}, {"coupling_planes", coupling_planes},
                 {"in_place", in_place},
-                {"fork_join", fork_join}};
+                {"fork_join", fork_join},
+                {"per_device", per_device}};
   for (const auto& c : checks)
     if (std::strcmp(argv[1], c.name) == 0) {
       c.run();

@@ -1,8 +1,9 @@
 """Host logic of the CUDA library's headers (buffers after a failed allocation,
-use of a caller's arrays, joining of two streams), compiled with the host
+use of a caller's arrays, joining of two streams, settings of a device), compiled with the host
 compiler against a fake CUDA runtime: no GPU, and no fault on one, is needed to
 see it."""
 import os
+import re
 import shutil
 import subprocess
 
@@ -28,7 +29,20 @@ def checks(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("name", ["mlp_growth", "coupling_planes", "in_place", "fork_join"])
+@pytest.mark.parametrize("name", ["mlp_growth", "coupling_planes", "in_place", "fork_join",
+                                  "per_device"])
 def test_host_state(checks, name):
     r = subprocess.run([checks, name], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_no_setting_of_a_device_is_made_once_per_process():
+    """A function-local static that asks for or sets something of the current
+    device would hold for the first device only."""
+    csrc = os.path.join(ROOT, "paper_1902_00095_gb300", "csrc")
+    for name in sorted(os.listdir(csrc)):
+        src = open(os.path.join(csrc, name)).read()
+        for m in re.finditer(r"static const [\w: ]+ \w+ = (?:\[[^;]*?\]\s*(?:\(\))?\s*\{.*?\n\s*\}"
+                             r"(?:\(\))?;|[^;\[]*;)", src, re.S):
+            assert not re.search(r"cudaFuncSetAttribute|cudaGetDevice\b|probe_\w+\(", m.group(0)), \
+                (name, m.group(0))
