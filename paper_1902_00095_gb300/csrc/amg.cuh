@@ -247,12 +247,26 @@ DevCSR csr_product(const DevCSR& A, const DevCSR& B, Pool& pool, Pool& scratch,
 void csr_product_numeric(const DevCSR& A, const DevCSR& B, const DevCSR& C, Pool& scratch,
                          cudaStream_t s);
 // Truncated (pmax >= 1 weights per row) classical or extended+i interpolation
-// P of level operator A (amg_interp.cu); P's arrays from `pool`. Returns false
-// when a row is past its capacities (nothing usable written).
-bool truncated_interpolation(const DevCSR& A, bool extended, int sms, const int* dpos,
-                             const unsigned char* strong, const signed char* state,
-                             const int* cidx, int nc, int pmax, Pool& pool, Pool& scratch,
-                             DevCSR& P, cudaStream_t s);
+// P of level operator A (amg_interp.cu); P's arrays from `pool`. Rows past its
+// capacities go through the untruncated form by a list.
+DevCSR truncated_interpolation(const DevCSR& A, bool extended, const int* dpos,
+                               const unsigned char* strong, const signed char* state,
+                               const int* cidx, int nc, int pmax, Pool& pool, Pool& scratch,
+                               cudaStream_t s);
+// whether to ask if a row of a level is past its capacities, and the answer
+// (device int: 1 when one is)
+bool interp_long_rows(const DevCSR& A);
+void rows_past_one_pass(const DevCSR& A, const unsigned char* strong, const signed char* state,
+                        int* past, cudaStream_t s);
+// Untruncated interpolation of the rows list[0, rows) of A (null: of all; row q
+// of the result is list[q]'s), and the pmax largest weights of such rows into
+// slots of pmax entries each (row i's at i * pmax, their number in cnt[i]).
+DevCSR untruncated_interpolation(const DevCSR& A, bool extended, const int* dpos,
+                                 const unsigned char* strong, const signed char* state,
+                                 const int* cidx, int nc, const int* list, int rows, Pool& pool,
+                                 Pool& scratch, cudaStream_t s);
+void truncate_listed_rows(const DevCSR& P, const int* list, int pmax, int* cnt, int* tcol,
+                          double* tval, cudaStream_t s);
 void csr_transpose_positions(const DevCSR& A, int* tpos, int* err, cudaStream_t s);
 
 }  // namespace tp

@@ -33,6 +33,13 @@ __device__ __forceinline__ bool nonzero_bits(double v) {
   return ((unsigned long long)__double_as_longlong(v) << 1) != 0;
 }
 
+// |w| as an ordered integer, NaN lowest
+__device__ __forceinline__ unsigned long long mag_key(double w) {
+  const unsigned long long m =
+      (unsigned long long)__double_as_longlong(w) & 0x7fffffffffffffffull;
+  return m <= 0x7ff0000000000000ull ? m + 1 : 0;
+}
+
 // index of key in a[lo, hi) (ascending), or -1
 __device__ __forceinline__ int find_in(const int* __restrict__ a, int lo, int hi, int key) {
   int h = hi;

@@ -3,9 +3,9 @@
 // nothing but the truncated row written to memory.
 //
 // The arithmetic and its order are those of the untruncated kernels followed by
-// k_trunc_fill (amg_setup.cu), which stay for untruncated interpolation and for
-// levels with a row past the largest capacities here, so the weights are the
-// same bit for bit.
+// k_trunc_fill (amg_setup.cu), which stay for untruncated interpolation, for the
+// rows past the largest capacities here and for levels of long rows that have
+// such a row, so the weights are the same bit for bit.
 //
 // What bounds it: the rows of the strong F neighbours have to be read (128
 // entries per F row on the first Galerkin level of the layered A_pp, 340 on the
@@ -50,11 +50,22 @@ struct InterpWork {
 // class's capacities go to the next class through a list. Levels of at most
 // kInterpFewRows rows that are not short start at the last class, a warp per
 // row: the others would leave most SMs without a warp.
-// The last class takes rows of up to 128 strong F neighbours (32 at a time): one
-// row past it sends its level to the untruncated kernels (at 32 neighbours the
-// channelised 128x128x64 system had one: 46.0 instead of 44.1 ms a step).
+// The last class takes rows of up to 128 strong F neighbours, 32 at a time.
 constexpr double kInterpShortMean = 20.0;
 constexpr int kInterpFewRows = 16384;
+// Levels of long rows on the mean are asked first whether a row is past the last
+// class (interp_long_rows, rows_past_one_pass), and go to the untruncated kernels
+// as a whole if one is: these wait for their longest rows, so the pass over the
+// others would come on top (random graph, levels of 4723 rows of 1164 entries and
+// of 963 of 907: 1.8 and 5.2 ms untruncated, the pass 0.6 and 1.5 ms more; setup
+// 28.9 -> 26.3 ms). Shorter levels are not asked: the pass is a small part of what
+// the untruncated kernels take there, and the few rows past it go to them by a
+// list (150000 rows of 23 entries, two of them with 800 strong F neighbours: 1.08
+// ms untruncated, 0.94 by pass and list; setup 34.4 -> 29.7 ms).
+constexpr int kInterpLongMean = 64;
+// the last class: strong F neighbours, entries, set members of a row, entries of
+// its neighbours' rows that count
+constexpr int kInterpKM = 128, kInterpRL = 1024, kInterpSet = 128, kInterpEnt = 1024;
 
 constexpr unsigned kAll = 0xffffffffu;
 constexpr unsigned char kSelf = 255;  // list entry a_ki (extended+i), no slot
@@ -97,9 +108,12 @@ __device__ __forceinline__ int hash_find(const int* hkey, int key) {
   return -1;
 }
 
-// key into the table (and, when new, onto the unordered set while it has room)
+// key into the table (and, when new, onto the unordered set while it has room);
+// a set past its capacity takes no more: its row goes elsewhere, and probes of a
+// filling table would cost more than the rest of the row
 template <int HS, int SET>
 __device__ __forceinline__ void hash_add(int* hkey, int* setc, int* ns, int key) {
+  if (*static_cast<volatile int*>(ns) > SET) return;
   unsigned h = hash_of<HS>(key);
   for (int p = 0; p < HS; ++p) {
     const int prev = atomicCAS(&hkey[h], -1, key);
@@ -112,13 +126,6 @@ __device__ __forceinline__ void hash_add(int* hkey, int* setc, int* ns, int key)
     h = (h + 1) & (unsigned)(HS - 1);
   }
   atomicAdd(ns, SET + 1);  // table full: overflow
-}
-
-// |w| as an ordered integer, NaN lowest
-__device__ __forceinline__ unsigned long long mag_key(double w) {
-  const unsigned long long m =
-      (unsigned long long)__double_as_longlong(w) & 0x7fffffffffffffffull;
-  return m <= 0x7ff0000000000000ull ? m + 1 : 0;
 }
 
 // EXT: extended+i, else classical. Rows list[0, *nlist) (list null: rows 0 to
@@ -241,6 +248,8 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp(
         };
         if (EXT) {
           for (int k0 = 0; k0 < nk_max; k0 += G) {
+            __syncwarp();
+            if (__all_sync(kAll, !act || s.ns[r] > SET)) break;
             if (k0 > 0) load(k0);
             for (int p0 = 0; p0 < total_max; p0 += G) {
               const int p = p0 + gl;
@@ -295,6 +304,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp(
         // the entries of the neighbours' rows that count, in order
         int ne = 0;
         for (int k0 = 0; k0 < nk_max; k0 += G) {
+          if (__all_sync(kAll, !act || over || ne > ENT)) break;
           if (nk_max > G) load(k0);
           const int ne0 = ne;
           int mine = 0;
@@ -490,6 +500,29 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp(
   }
 }
 
+// sets *past when an F row has more entries, strong F neighbours or strong C
+// neighbours (its classical set, a part of its extended+i one) than the last class
+// holds, or, if the level's entries (a share `fill` of n^2) lie evenly, more
+// entries of the neighbours' rows in the set (a warp per row)
+__global__ void k_rows_past(int n, float fill, const int* __restrict__ rp,
+                            const int* __restrict__ col,
+                            const unsigned char* __restrict__ strong,
+                            const signed char* __restrict__ state, int* __restrict__ past) {
+  const int i = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
+  if (i >= n || state[i] == kC) return;
+  const int r0 = rp[i], r1 = rp[i + 1];
+  int nk = 0, ns = 0;
+  if (r1 - r0 <= kInterpRL)
+    for (int e = r0 + lane; e < r1; e += 32)
+      if (strong[e]) (state[col[e]] == kC ? ns : nk) += 1;
+  nk = __reduce_add_sync(kAll, nk);
+  ns = __reduce_add_sync(kAll, ns);
+  if (lane == 0 && (r1 - r0 > kInterpRL || nk > kInterpKM || ns > kInterpSet ||
+                    fill * (float)nk * (float)ns > (float)kInterpEnt))
+    *past = 1;
+}
+
 // rows of at most pmax entries at i * pmax to the compact CSR
 __global__ void k_interp_compact(int n, int pmax, const int* __restrict__ tcol,
                                  const double* __restrict__ tval, const int* __restrict__ Prp,
@@ -543,17 +576,28 @@ void interp_tiers(const DevCSR& A, int sms, const int* dpos, const unsigned char
     list = w.olist1;
     nlist = w.ocnt + 1;
   }
-  launch_tier<EXT, 32, 1, 128, 1024, 128, 1024, 2>(6, sms, n, list, nlist, A, dpos, strong, state,
-                                                  cidx, pmax, w.cnt, w.tcol, w.tval, w.olist0,
-                                                  w.ocnt + 2, s);
+  launch_tier<EXT, 32, 1, kInterpSet, kInterpEnt, kInterpKM, kInterpRL, 2>(
+      6, sms, n, list, nlist, A, dpos, strong, state, cidx, pmax, w.cnt, w.tcol, w.tval, w.olist0,
+      w.ocnt + 2, s);
 }
 
 }  // namespace
 
-bool truncated_interpolation(const DevCSR& A, bool extended, int sms, const int* dpos,
-                             const unsigned char* strong, const signed char* state,
-                             const int* cidx, int nc, int pmax, Pool& pool, Pool& scratch,
-                             DevCSR& P, cudaStream_t s) {
+bool interp_long_rows(const DevCSR& A) { return A.nnz > (long long)kInterpLongMean * A.n; }
+
+void rows_past_one_pass(const DevCSR& A, const unsigned char* strong, const signed char* state,
+                        int* past, cudaStream_t s) {
+  TP_CUDA_TRY(cudaMemsetAsync(past, 0, sizeof(int), s));
+  const float fill = (float)((double)A.nnz / ((double)A.n * A.n));
+  k_rows_past<<<grid_for((long long)A.n * 32), kBlock, 0, s>>>(A.n, fill, A.rowptr, A.col, strong,
+                                                              state, past);
+  TP_LAUNCH_CHECK();
+}
+
+DevCSR truncated_interpolation(const DevCSR& A, bool extended, const int* dpos,
+                               const unsigned char* strong, const signed char* state,
+                               const int* cidx, int nc, int pmax, Pool& pool, Pool& scratch,
+                               cudaStream_t s) {
   const int n = A.n;
   InterpWork w;
   w.cnt = scratch.alloc<int>(n + 1);
@@ -562,21 +606,27 @@ bool truncated_interpolation(const DevCSR& A, bool extended, int sms, const int*
   w.olist0 = scratch.alloc<int>(n);
   w.olist1 = scratch.alloc<int>(n);
   w.ocnt = scratch.alloc<int>(3);
-  if (extended) interp_tiers<true>(A, sms, dpos, strong, state, cidx, pmax, w, s);
-  else interp_tiers<false>(A, sms, dpos, strong, state, cidx, pmax, w, s);
+  if (extended) interp_tiers<true>(A, device_sms(), dpos, strong, state, cidx, pmax, w, s);
+  else interp_tiers<false>(A, device_sms(), dpos, strong, state, cidx, pmax, w, s);
   int over = 0;  // rows past the last capacities
+  DevCSR P;
   P.n = n;
   P.m = nc;
   P.rowptr = pool.alloc<int>(n + 1);
-  const long long total = scan_exclusive(w.cnt, P.rowptr, n, scratch, s, w.ocnt + 2, &over);
-  if (over > 0) return false;
+  long long total = scan_exclusive(w.cnt, P.rowptr, n, scratch, s, w.ocnt + 2, &over);
+  if (over > 0) {
+    const DevCSR U = untruncated_interpolation(A, extended, dpos, strong, state, cidx, nc,
+                                               w.olist0, over, scratch, scratch, s);
+    truncate_listed_rows(U, w.olist0, pmax, w.cnt, w.tcol, w.tval, s);
+    total = scan_exclusive(w.cnt, P.rowptr, n, scratch, s);
+  }
   P.nnz = (int)total;
   P.col = pool.alloc<int>(P.nnz + 1);
   P.val = pool.alloc<double>(P.nnz + 1);
   k_interp_compact<<<grid_for((long long)n * pmax), kBlock, 0, s>>>(n, pmax, w.tcol, w.tval,
                                                                     P.rowptr, P.col, P.val);
   TP_LAUNCH_CHECK();
-  return true;
+  return P;
 }
 
 }  // namespace tp

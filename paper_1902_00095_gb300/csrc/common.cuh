@@ -159,7 +159,7 @@ long long scan_exclusive(const int* in, int* out, int n, Pool& scratch, cudaStre
                          const int* extra = nullptr, int* extra_host = nullptr);
 // the same over 1 where state[i] == what, else 0
 long long scan_states(const signed char* state, signed char what, int* out, int n, Pool& scratch,
-                      cudaStream_t s);
+                      cudaStream_t s, const int* extra = nullptr, int* extra_host = nullptr);
 
 // Deterministic sum of n doubles (fixed block partition and tree order),
 // result in *out (device).

@@ -216,8 +216,8 @@ long long scan_exclusive(const int* in, int* out, int n, Pool& scratch, cudaStre
 }
 
 long long scan_states(const signed char* state, signed char what, int* out, int n, Pool& scratch,
-                      cudaStream_t s) {
-  return scan_values(ScanStates{state, what}, out, n, scratch, s, nullptr, nullptr);
+                      cudaStream_t s, const int* extra, int* extra_host) {
+  return scan_values(ScanStates{state, what}, out, n, scratch, s, extra, extra_host);
 }
 
 void sum_fixed(const double* x, int n, double* out, double* partials, int nparts, cudaStream_t s) {
