@@ -170,8 +170,8 @@ bool usable_in_place(int device, const T* p, size_t n) {
 }
 
 // A training batch on the device: the caller's device arrays as they are, or
-// the host arrays in one copy through a pinned image (five copies from pageable
-// memory, each staged by the runtime, took half of a step on 4096 samples).
+// the host arrays in one copy through a pinned image where they are short
+// (MlpStage::kImageMax), else in five copies.
 struct MlpBatch {
   const float* X;
   const double *St, *Sd, *target;
@@ -194,9 +194,10 @@ MlpBatch mlp_batch(tp_mlp* a, int B, const float* X, const int* slot, const doub
     const void* from;
   } part[5] = {{oSt, nd, St}, {oSd, nd, Sd}, {oT, nd, target}, {oX, nX, X}, {oS, n * sizeof(int), slot}};
   char* d = a->stage.batch;
-  if (ptr_is_device) {
+  if (ptr_is_device || B > tp::MlpStage::kImageMax) {
+    const cudaMemcpyKind kind = ptr_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     for (const auto& q : part)
-      TP_CUDA_TRY(cudaMemcpyAsync(d + q.at, q.from, q.bytes, cudaMemcpyDeviceToDevice, a->s));
+      TP_CUDA_TRY(cudaMemcpyAsync(d + q.at, q.from, q.bytes, kind, a->s));
   } else {
     char* h = a->stage.host_image();
     for (const auto& q : part) std::memcpy(h + q.at, q.from, q.bytes);

@@ -110,7 +110,8 @@ static void mlp_growth() {
     CHECK(inside(g_device, st.batch, n * tp::MlpStage::kBatchBytes));
     CHECK(inside(g_device, st.O, n * tp::kMlpOut * sizeof(float)));
     CHECK(inside(g_device, st.partials, (n + 15) / 16 * tp::kMlpPartial * sizeof(float)));
-    CHECK(inside(g_pinned, st.host_image(), n * tp::MlpStage::kBatchBytes));
+    CHECK(inside(g_pinned, st.host_image(),
+                 tp::MlpStage::kImageMax * tp::MlpStage::kBatchBytes));
   }
   CHECK(g_device.empty() && g_pinned.empty());
 }
