@@ -31,10 +31,15 @@ constexpr int kDotWideU = 2, kDotNarrowU = 4;  // elements a thread loads at a t
 constexpr long long kDotWideMaxN = 1ll << 20;  // vector length up to which 8 are taken
 // An iteration is enqueued before the host has seen the previous one's residual
 // estimate only while the last estimate it has seen is more than this factor
-// above the tolerance. Iterations reduce it 3- to 15-fold, so the last one is
-// not run ahead of and thrown away (an eighteenth iteration of 6.5 ms on the
-// layered 256x256x64 system, a fourteenth of 0.8 ms at 64x64x32), for a wait of
-// some 10 us at each of the last few.
+// above the tolerance, so that the last one is not run ahead of and thrown away
+// (an eighteenth iteration of 6.5 ms on the layered 256x256x64 system, a
+// fourteenth of 0.8 ms at 64x64x32), for a wait of some 10 us at each of the last
+// few. Iterations reduce the estimate by 1.2 to 15, some 2.5 on average on the
+// large systems; solve times with the factor at 1 (always ahead) / 20 / 400 /
+// never ahead: 14 iterations at 64x64x32 10.7 / 10.0 / 10.0 / 10.1 ms, 9 at
+// 16x16x8 1.84 / 1.67 / 1.68 / 1.70, and for slowly converging solves 95 at
+// 32x32x16 (a reduction of 1.2) 23.9 / 23.5 / 23.5 / 23.8, 89 at 64x64x32
+// 63.2 / 62.6 / 62.7 / 62.9.
 constexpr double kRunAhead = 20.0;
 // Schur columns solved side by side, on grids of up to kColumnLaneRows cells
 // (beyond, one solve fills the GPU and a workspace is large)
@@ -111,11 +116,13 @@ __global__ void k_rhs_minus(int N, const int* __restrict__ rp, const int* __rest
 // the same with the plane stored by grid direction (launch_coupling_planes):
 // coalesced loads, no column indices, the row's values loaded before the
 // dependency wait (the planes do not change during a solve). An absent
-// neighbour's value is 0 and its column is the row's own; the sum runs in the
-// CSR row's order. Bound by HBM (80 bytes per row, 50 us at 4.2 M rows); from
-// the CSR plane, one thread per row striding over its entries, it took 76 us
-// after the V-cycle before it ended. The layered 256x256x64 solve (two per
-// iteration) 113.7 -> 112.9 ms.
+// neighbour's value is 0 and its column, the row plus the slot's offset (the row
+// itself outside [0, N)), is some other cell's: it adds an exact zero while x is
+// finite. A non-finite x reaches a cell more than from CSR, in a solve that has
+// broken down by then. The sum runs in the CSR row's order. Bound by HBM (80 bytes
+// per row, 50 us at 4.2 M rows); from the CSR plane, one thread per row striding
+// over its entries, it took 76 us after the V-cycle before it ended. The layered
+// 256x256x64 solve (two per iteration) 113.7 -> 112.9 ms.
 __global__ void __launch_bounds__(256) k_rhs_minus_grid(int N, int nx, int nxy,
                                                         const double* __restrict__ plane,
                                                         const double* __restrict__ b,
