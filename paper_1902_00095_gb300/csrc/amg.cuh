@@ -254,7 +254,7 @@ DevCSR truncated_interpolation(const DevCSR& A, bool extended, const int* dpos,
                                const int* cidx, int nc, int pmax, Pool& pool, Pool& scratch,
                                cudaStream_t s);
 // whether to ask if a row of a level is past its capacities, and the answer
-// (device int: 1 when one is)
+// (device int, 0 before: 1 when one is)
 bool interp_long_rows(const DevCSR& A);
 void rows_past_one_pass(const DevCSR& A, const unsigned char* strong, const signed char* state,
                         int* past, cudaStream_t s);

@@ -58,11 +58,11 @@ constexpr int kInterpFewRows = 16384;
 // as a whole if one is: these wait for their longest rows, so the pass over the
 // others would come on top (random graph, levels of 4723 rows of 1164 entries and
 // of 963 of 907: 1.8 and 5.2 ms untruncated, the pass 0.6 and 1.5 ms more; setup
-// 28.9 -> 26.3 ms). Shorter levels are not asked: the pass is a small part of what
-// the untruncated kernels take there, and the few rows past it go to them by a
-// list (150000 rows of 23 entries, two of them with 800 strong F neighbours: 1.08
-// ms untruncated, 0.94 by pass and list; setup 34.4 -> 29.7 ms).
-constexpr int kInterpLongMean = 64;
+// 28.9 -> 26.3 ms). Shorter levels, a grid's among them, are not asked: the pass is
+// a small part of what the untruncated kernels take there, and the few rows past
+// it go to them by a list (150000 rows of 23 entries, two of them with 800 strong F
+// neighbours: 1.08 ms untruncated, 0.94 by pass and list; setup 34.5 -> 29.4 ms).
+constexpr int kInterpLongMean = 100;
 // the last class: strong F neighbours, entries, set members of a row, entries of
 // its neighbours' rows that count
 constexpr int kInterpKM = 128, kInterpRL = 1024, kInterpSet = 128, kInterpEnt = 1024;
@@ -108,12 +108,9 @@ __device__ __forceinline__ int hash_find(const int* hkey, int key) {
   return -1;
 }
 
-// key into the table (and, when new, onto the unordered set while it has room);
-// a set past its capacity takes no more: its row goes elsewhere, and probes of a
-// filling table would cost more than the rest of the row
+// key into the table (and, when new, onto the unordered set while it has room)
 template <int HS, int SET>
 __device__ __forceinline__ void hash_add(int* hkey, int* setc, int* ns, int key) {
-  if (*static_cast<volatile int*>(ns) > SET) return;
   unsigned h = hash_of<HS>(key);
   for (int p = 0; p < HS; ++p) {
     const int prev = atomicCAS(&hkey[h], -1, key);
@@ -248,8 +245,6 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp(
         };
         if (EXT) {
           for (int k0 = 0; k0 < nk_max; k0 += G) {
-            __syncwarp();
-            if (__all_sync(kAll, !act || s.ns[r] > SET)) break;
             if (k0 > 0) load(k0);
             for (int p0 = 0; p0 < total_max; p0 += G) {
               const int p = p0 + gl;
@@ -304,7 +299,6 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp(
         // the entries of the neighbours' rows that count, in order
         int ne = 0;
         for (int k0 = 0; k0 < nk_max; k0 += G) {
-          if (__all_sync(kAll, !act || over || ne > ENT)) break;
           if (nk_max > G) load(k0);
           const int ne0 = ne;
           int mine = 0;
@@ -587,7 +581,6 @@ bool interp_long_rows(const DevCSR& A) { return A.nnz > (long long)kInterpLongMe
 
 void rows_past_one_pass(const DevCSR& A, const unsigned char* strong, const signed char* state,
                         int* past, cudaStream_t s) {
-  TP_CUDA_TRY(cudaMemsetAsync(past, 0, sizeof(int), s));
   const float fill = (float)((double)A.nnz / ((double)A.n * A.n));
   k_rows_past<<<grid_for((long long)A.n * 32), kBlock, 0, s>>>(A.n, fill, A.rowptr, A.col, strong,
                                                               state, past);

@@ -1574,13 +1574,12 @@ void Hierarchy::setup(const DevCSR& A0, const AmgOpts& o, cudaStream_t s) {
     int* cidx = scratch.alloc<int>(n + 1);
     // (one-pass interpolation: whether a row of a long-row level cannot take it
     // comes back with the number of C points)
-    int* past = nullptr;
+    const bool ask = opts.pmax > 0 && interp_long_rows(A);
+    int* past = undecided;  // 0 by now
     int rows_past = 0;
-    if (opts.pmax > 0 && interp_long_rows(A)) {
-      past = scratch.alloc<int>(1);
-      rows_past_one_pass(A, cur.strong, cur.cf, past, s);
-    }
-    const int nc = (int)scan_states(cur.cf, kC, cidx, n, scratch, s, past, &rows_past);
+    if (ask) rows_past_one_pass(A, cur.strong, cur.cf, past, s);
+    const int nc = (int)scan_states(cur.cf, kC, cidx, n, scratch, s, ask ? past : nullptr,
+                                    &rows_past);
     if (nc == 0 || (double)nc > 0.9 * (double)n) {
       cur.cf = nullptr;  // this level becomes the coarsest
       break;
