@@ -7,6 +7,7 @@
 #include "fork_join.cuh"
 #include "in_place.cuh"
 #include "mlp_stage.cuh"
+#include "per_device.cuh"
 #include "solver.cuh"
 
 using tp::Error;
@@ -166,7 +167,7 @@ bool usable_in_place(int device, const T* p, size_t n) {
       cudaGetLastError();
     return reinterpret_cast<tp::PointerQuery>(f);
   }();
-  return tp::usable_in_place(query, device, p, n);
+  return tp::usable_in_place(query, tp::device_count(), device, p, n);
 }
 
 // A training batch on the device: the caller's device arrays as they are, or
@@ -1125,7 +1126,7 @@ int assemble_device(tp_ctx* c, double dt) {
 void extract_blocks(tp_ctx* c) {
   launch_extract_blocks(c->nnzb, c->bval, c->App, c->ApT, c->ATp, c->ATT, c->s);
   if (c->grid.nx < 2 || c->grid.ny < 2 || c->grid.nz < 2) return;
-  if (c->planes.ensure(c->N))
+  if (c->planes.ensure(c->N, c->pool))
     launch_coupling_planes(c->grid, c->rowptr, c->bval, c->planes.ApT, c->planes.ATp, c->s);
 }
 
@@ -1293,7 +1294,7 @@ bool give_back(tp_ctx* c) {
     drop_column_lanes(c);
     return true;
   }
-  if (!c->planes.ApT) return false;
+  if (!c->planes.owned()) return false;
   TP_CUDA_TRY(cudaStreamSynchronize(c->s));
   const bool recorded = c->pc_graph != nullptr;  // it reads the planes
   drop_graph(c);

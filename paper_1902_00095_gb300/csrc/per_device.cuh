@@ -5,6 +5,15 @@
 
 namespace tp {
 
+// devices that the process sees, at least 2 if the runtime cannot tell
+inline int device_count() {
+  static const int n = [] {
+    int d = 0;
+    return cudaGetDeviceCount(&d) == cudaSuccess ? d : 2;
+  }();
+  return n;
+}
+
 // make()'s value for the current device, made at the first call on it: kernel
 // attributes and SM counts belong to a device, and a process may have contexts
 // of the library on several. Safe with several threads; a make() that throws is
@@ -14,8 +23,8 @@ class PerDevice {
  public:
   template <class F>
   T operator()(F make) {
-    int dev = 0;
-    TP_CUDA_TRY(cudaGetDevice(&dev));
+    int dev = 0;  // asked for where there is a choice: every launch of some kernels comes by
+    if (device_count() != 1) TP_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kMax) return make();
     std::call_once(flag_[dev], [&] { value_[dev] = make(); });
     return value_[dev];

@@ -11,14 +11,18 @@ struct CouplingPlanes {
   double *ApT = nullptr, *ATp = nullptr;
   bool refused = false;  // no memory when last asked for (cleared by a build)
   Pool pool;
+  // planes of up to this many bytes come from the context's pool and stay there
+  // (an allocation of their own takes some 50 us of a new context's first build)
+  static constexpr size_t kShared = size_t(4) << 20;
 
   // both planes of N cells, or neither (false)
-  bool ensure(size_t N) {
+  bool ensure(size_t N, Pool& shared) {
     if (ApT) return true;
     if (refused) return false;
     const size_t each = (7 * N + 31) / 32 * 32;
     try {
-      double* p = pool.alloc<double>(2 * each);
+      Pool& from = 2 * each * sizeof(double) <= kShared ? shared : pool;
+      double* p = from.alloc<double>(2 * each);
       ApT = p;
       ATp = p + each;
     } catch (const Error& e) {
@@ -28,7 +32,9 @@ struct CouplingPlanes {
     }
     return true;
   }
-  // for an allocation that cannot be done without; nothing may be reading them
+  // memory of their own, which give_back() frees for an allocation that cannot be
+  // done without; nothing may be reading them
+  bool owned() const { return pool.reserved() > 0; }
   void give_back() {
     ApT = ATp = nullptr;
     refused = true;

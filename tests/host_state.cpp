@@ -44,6 +44,10 @@ cudaError_t cudaFreeHost(void* p) {
   return cudaSuccess;
 }
 static int g_dev = 0, g_attributes = 0;
+cudaError_t cudaGetDeviceCount(int* n) {
+  *n = 4;
+  return cudaSuccess;
+}
 cudaError_t cudaGetDevice(int* d) {
   *d = g_dev;
   return cudaSuccess;
@@ -119,18 +123,21 @@ static void mlp_growth() {
 // memory for one plane but not for two: neither is there, now and when asked
 // again, and both once there is room after a build
 static void coupling_planes() {
-  const size_t N = 1000001;
-  {
+  for (size_t N : {size_t(1001), size_t(1000001)}) {
     tp::CouplingPlanes p;
-    g_device_limit = 7 * N * sizeof(double) + (4u << 20);
-    CHECK(!p.ensure(N) && !p.ApT && !p.ATp);
+    tp::Pool shared;
+    shared.alloc<char>(1);
+    if (N < 5000) shared.alloc<char>(shared.reserved() - 7 * N * sizeof(double) - 512);
+    g_device_limit = g_device_used + 7 * N * sizeof(double);
+    if (N < 5000) g_device_limit = g_device_used;
+    CHECK(!p.ensure(N, shared) && !p.ApT && !p.ATp);
     g_device_limit = ~size_t(0);
-    CHECK(!p.ensure(N) && !p.ApT && !p.ATp);
+    CHECK(!p.ensure(N, shared) && !p.ApT && !p.ATp);
     p.refused = false;
-    CHECK(p.ensure(N));
+    CHECK(p.ensure(N, shared));
     CHECK(inside(g_device, p.ApT, 7 * N * sizeof(double)));
     CHECK(inside(g_device, p.ATp, 7 * N * sizeof(double)));
-    CHECK(p.ATp >= p.ApT + 7 * N);
+    CHECK(p.ATp >= p.ApT + 7 * N && p.owned() == (N > 5000));
   }
   CHECK(g_device.empty());
 }
@@ -153,7 +160,7 @@ static CUresult fake_query(unsigned n, CUpointer_attribute* what, void** to, CUd
 static void in_place() {
   const char* base = reinterpret_cast<char*>(size_t(1) << 40);
   auto usable = [&](int device, size_t byte, size_t n) {
-    return tp::usable_in_place(fake_query, device, reinterpret_cast<const double*>(base + byte), n);
+    return tp::usable_in_place(fake_query, 2, device, reinterpret_cast<const double*>(base + byte), n);
   };
   g_type = CU_MEMORYTYPE_DEVICE;
   g_owner = 1;
@@ -163,9 +170,11 @@ static void in_place() {
   CHECK(!usable(1, 4, 1));                           // unaligned
   g_owner = 0;
   CHECK(usable(0, 0, 512) && !usable(1, 0, 512));
+  const double* p = reinterpret_cast<const double*>(base);
+  CHECK(tp::usable_in_place(fake_query, 1, 0, p, 512) && !tp::usable_in_place(fake_query, 1, 0, p, 513));
   g_type = CU_MEMORYTYPE_HOST;
-  CHECK(!usable(0, 0, 1));
-  CHECK(!tp::usable_in_place<double>(nullptr, 0, nullptr, 1));
+  CHECK(!usable(0, 0, 1) && !tp::usable_in_place(fake_query, 1, 0, p, 1));
+  CHECK(!tp::usable_in_place<double>(nullptr, 1, 0, nullptr, 1));
 }
 
 // the first stream waits for the second's work however the two sides end, and
